@@ -131,7 +131,7 @@ struct Blob {
 template <class T> const T* at(void* base, size_t off) { return reinterpret_cast<const T*>(static_cast<unsigned char*>(base) + off); }
 
 // 16-byte device values of a precision: complex double, or complex double-float
-// (each part split into hi = float(x), lo = float(x - hi))
+// (each part split into hi = float(x), lo = float(x - hi): re.hi, im.hi, re.lo, im.lo)
 struct Val16 { unsigned char b[16]; };
 std::vector<Val16> to_val(const std::vector<cplx>& v, int prec) {
     std::vector<Val16> o(v.size());
@@ -142,8 +142,8 @@ std::vector<Val16> to_val(const std::vector<cplx>& v, int prec) {
         } else {
             float x[4];
             const double re = v[i].real(), im = v[i].imag();
-            x[0] = (float)re; x[1] = (float)(re - (double)x[0]);
-            x[2] = (float)im; x[3] = (float)(im - (double)x[2]);
+            x[0] = (float)re; x[2] = (float)(re - (double)x[0]);
+            x[1] = (float)im; x[3] = (float)(im - (double)x[1]);
             std::memcpy(o[i].b, x, 16);
         }
     }

@@ -212,10 +212,7 @@ __device__ __forceinline__ void stage_site_df(const double* __restrict__ U, cons
     eD = exponent_of(md);
     if (i < 288) {
         const double sc = pow2d(-(i < 144 ? eU : eD));
-        cdf z;
-        z.re = df_from_double(v.x * sc);
-        z.im = df_from_double(v.y * sc);
-        q[i] = z;
+        q[i] = cdf_make(df_from_double(v.x * sc), df_from_double(v.y * sc));
     }
 }
 
@@ -320,8 +317,7 @@ __global__ void __launch_bounds__(kThreads) block_project_df_kernel(BlockDev b, 
             if (k < 0) k += L;
             double sn, cs;
             sincospi(-2.0 * (double)k / (double)L, &sn, &cs);
-            ph_s.re = df_from_double(cs);
-            ph_s.im = df_from_double(sn);
+            ph_s = cdf_make(df_from_double(cs), df_from_double(sn));
         }
         __syncthreads();
         diquarks_df(b.n_types, ty, q, dq);
@@ -333,8 +329,7 @@ __global__ void __launch_bounds__(kThreads) block_project_df_kernel(BlockDev b, 
             cdf v = block_entry_df(ty, code, q, dq);
             if (mom) v = MIXED::mul(v, ph);
             const float sc = ty[code >> 16].q1 ? sc1 : sc0;
-            v.re.hi *= sc; v.re.lo *= sc; v.im.hi *= sc; v.im.lo *= sc;
-            acc[f] = MIXED::vadd(acc[f], v);
+            acc[f] = MIXED::vadd(acc[f], cdf_scale(v, sc));
         }
     }
     cd* o = part + (slice * tiles + tile) * (int64_t)b.n_f + f0;
@@ -342,7 +337,7 @@ __global__ void __launch_bounds__(kThreads) block_project_df_kernel(BlockDev b, 
     for (int f = threadIdx.x; f < nf; f += blockDim.x) {
         const cdf v = acc[f];
         const double sc = ty[entry_code(b, f0 + f) >> 16].q1 ? s1 : s0;
-        o[f] = cd_make(df_to_double(v.re) * sc, df_to_double(v.im) * sc);
+        o[f] = cd_make(df_to_double(cdf_re(v)) * sc, df_to_double(cdf_im(v)) * sc);
     }
 }
 
@@ -427,10 +422,7 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
     const double sc = pow2d(-max(min(e, 1000), -1000));
     for (int i = threadIdx.x; i < t.n_f; i += blockDim.x) {
         const cd v = Fg[i];
-        cdf z;
-        z.re = df_from_double(v.re * sc);
-        z.im = df_from_double(v.im * sc);
-        fs[i] = z;
+        fs[i] = cdf_make(df_from_double(v.re * sc), df_from_double(v.im * sc));
     }
     __syncthreads();
     const int np = t.A - 1;
@@ -446,10 +438,8 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
             const float2 w = __ldg(t.leaf_w + l);
             const cdf f = fs[__ldg(t.leaf_f + l)];
             // (w.x + i w.y) f with float weights (exact products by error-free transformation)
-            dacc_fma_f(a.r0, w.x, f.re);
-            dacc_fma_f(a.r1, -w.y, f.im);
-            dacc_fma_f(a.i0, w.x, f.im);
-            dacc_fma_f(a.i1, w.y, f.re);
+            dacc2_fma_f(a.x, w.x, f);
+            dacc2_fma_f(a.y, w.y, f);
         }
         MIXED::add(tot, MIXED::mul(pre, MIXED::get(a)));
     }

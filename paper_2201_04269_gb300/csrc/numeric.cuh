@@ -8,6 +8,12 @@
 //        rounded value itself is part of an error-free transformation, so the compiler
 //        never fuses those operations.
 // Accumulators keep an unnormalised (hi, lo) pair and are renormalised once at the end.
+// Complex double-float values are held as the packed pairs (re.hi, im.hi), (re.lo, im.lo) and
+// every error-free transformation runs on both parts at once with f32x2 instructions: two
+// FP32 operations per issue slot at the same FMA-pipe rate (FFMA 3.9, FFMA2 1.99 warp
+// instructions per cycle and SM, measured), each rounded as the scalar one.  Broadcast and
+// swapped operands of a pair cost no instruction; negating a pair does, so differences are
+// multiply-adds with -1 (one rounding, exact product).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -18,7 +24,8 @@ struct cd { double re, im; };
 struct __align__(32) d4 { double x, y, z, w; };
 __host__ __device__ __forceinline__ d4 make_d4(double x, double y, double z, double w) { d4 r; r.x = x; r.y = y; r.z = z; r.w = w; return r; }
 struct df { float hi, lo; };
-struct cdf { df re, im; };
+typedef unsigned long long f32x2;                 // two floats, first in the low half
+struct __align__(16) cdf { f32x2 h, l; };         // (re.hi, im.hi), (re.lo, im.lo)
 
 __host__ __device__ __forceinline__ cd cd_make(double r, double i) { cd z; z.re = r; z.im = i; return z; }
 
@@ -61,41 +68,95 @@ __device__ __forceinline__ df df_div(df x, df y) {
     return fast_two_sum(q1, q2);
 }
 
-// unnormalised accumulator
-struct dacc { float hi, lo; };
-__device__ __forceinline__ void dacc_zero(dacc& a) { a.hi = 0.f; a.lo = 0.f; }
-// a += x * y
-__device__ __forceinline__ void dacc_fma(dacc& a, df x, df y) {
-    float p = __fmul_rn(x.hi, y.hi);
-    float e = fmaf(x.hi, y.hi, -p);
-    e = fmaf(x.hi, y.lo, e);
-    e = fmaf(x.lo, y.hi, e);
-    float s = __fadd_rn(a.hi, p);
-    float bp = __fsub_rn(s, a.hi);
-    float t = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bp)), __fsub_rn(p, bp));
-    a.hi = s;
-    a.lo = __fadd_rn(a.lo, __fadd_rn(t, e));
+// ------------------------------------------------------------------ packed pairs
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
 }
-// a += w * x with a float w (exact: w has no low part)
-__device__ __forceinline__ void dacc_fma_f(dacc& a, float w, df x) {
-    float p = __fmul_rn(x.hi, w);
-    float e = fmaf(x.hi, w, -p);
-    e = fmaf(x.lo, w, e);
-    float s = __fadd_rn(a.hi, p);
-    float bp = __fsub_rn(s, a.hi);
-    float t = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bp)), __fsub_rn(p, bp));
-    a.hi = s;
-    a.lo = __fadd_rn(a.lo, __fadd_rn(t, e));
+__device__ __forceinline__ float2 up2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
 }
-// a += x
-__device__ __forceinline__ void dacc_add(dacc& a, df x) {
-    float s = __fadd_rn(a.hi, x.hi);
-    float bp = __fsub_rn(s, a.hi);
-    float t = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bp)), __fsub_rn(x.hi, bp));
-    a.hi = s;
-    a.lo = __fadd_rn(a.lo, __fadd_rn(t, x.lo));
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
-__device__ __forceinline__ df dacc_get(const dacc& a) { return fast_two_sum(a.hi, a.lo); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pk2(-1.f, -1.f), a); }
+
+struct df2 { f32x2 hi, lo; };                     // a double-float per part
+__device__ __forceinline__ df2 fast_two_sum2(f32x2 a, f32x2 b) {
+    df2 r;
+    r.hi = add2(a, b);
+    r.lo = sub2(b, sub2(r.hi, a));
+    return r;
+}
+__device__ __forceinline__ df2 df_add2(df2 a, df2 b) {
+    const f32x2 s = add2(a.hi, b.hi), bp = sub2(s, a.hi);
+    const f32x2 e = add2(sub2(a.hi, sub2(s, bp)), sub2(b.hi, bp));
+    return fast_two_sum2(s, add2(e, add2(a.lo, b.lo)));
+}
+
+// unnormalised accumulator of both parts
+struct dacc2 { f32x2 hi, lo; };
+// a += p + e with p given as its negative (TwoSum of a.hi and p)
+__device__ __forceinline__ void dacc2_sum(dacc2& a, f32x2 np, f32x2 e) {
+    const f32x2 s = sub2(a.hi, np), bp = sub2(s, a.hi);
+    const f32x2 t = sub2(sub2(a.hi, sub2(s, bp)), add2(np, bp));
+    a.hi = s;
+    a.lo = add2(a.lo, add2(t, e));
+}
+// a += x * y for a real double-float x and both parts of y
+__device__ __forceinline__ void dacc2_fma(dacc2& a, float xh, float xl, const cdf& y) {
+    const f32x2 x = pk2(xh, xh);
+    const f32x2 np = mul2(pk2(-xh, -xh), y.h);
+    f32x2 e = fma2(x, y.h, np);
+    e = fma2(x, y.l, e);
+    e = fma2(pk2(xl, xl), y.h, e);
+    dacc2_sum(a, np, e);
+}
+// a += w * y with a float w (exact: w has no low part)
+__device__ __forceinline__ void dacc2_fma_f(dacc2& a, float w, const cdf& y) {
+    const f32x2 x = pk2(w, w);
+    const f32x2 np = mul2(pk2(-w, -w), y.h);
+    f32x2 e = fma2(x, y.h, np);
+    e = fma2(x, y.l, e);
+    dacc2_sum(a, np, e);
+}
+// a += y
+__device__ __forceinline__ void dacc2_add(dacc2& a, const cdf& y) {
+    const f32x2 s = add2(a.hi, y.h), bp = sub2(s, a.hi);
+    const f32x2 t = add2(sub2(a.hi, sub2(s, bp)), sub2(y.h, bp));
+    a.hi = s;
+    a.lo = add2(a.lo, add2(t, y.l));
+}
+__device__ __forceinline__ cdf cdf_make(df re, df im) {
+    cdf z;
+    z.h = pk2(re.hi, im.hi);
+    z.l = pk2(re.lo, im.lo);
+    return z;
+}
+__device__ __forceinline__ df cdf_re(const cdf& z) { df r; r.hi = up2(z.h).x; r.lo = up2(z.l).x; return r; }
+__device__ __forceinline__ df cdf_im(const cdf& z) { df r; r.hi = up2(z.h).y; r.lo = up2(z.l).y; return r; }
+// both parts times a power of two
+__device__ __forceinline__ cdf cdf_scale(const cdf& z, float p) {
+    cdf r;
+    r.h = mul2(z.h, pk2(p, p));
+    r.l = mul2(z.l, pk2(p, p));
+    return r;
+}
 
 // ------------------------------------------------------------------ precision traits
 // Each trait provides: value type V (complex), accumulator A, and
@@ -163,78 +224,71 @@ struct FP64 {
 
 struct MIXED {
     typedef cdf V;
-    // four independent chains (re: +x.re y.re and -x.im y.im; im: x.re y.im and x.im y.re)
-    // so that consecutive multiply-adds do not wait on each other
-    struct A { dacc r0, r1, i0, i1; };
+    // two independent chains: x = sum of x.re y, y = sum of x.im y; the value is
+    // (x.re - y.im, x.im + y.re)
+    struct A { dacc2 x, y; };
     static constexpr int kind = 1;
-    __device__ __forceinline__ static V zero() { V z; z.re.hi = z.re.lo = z.im.hi = z.im.lo = 0.f; return z; }
-    __device__ __forceinline__ static V one() { V z = zero(); z.re.hi = 1.f; return z; }
-    __device__ __forceinline__ static void acc_zero(A& a) { dacc_zero(a.r0); dacc_zero(a.r1); dacc_zero(a.i0); dacc_zero(a.i1); }
+    __device__ __forceinline__ static V zero() { V z; z.h = z.l = 0ull; return z; }
+    __device__ __forceinline__ static V one() { V z = zero(); z.h = pk2(1.f, 0.f); return z; }
+    __device__ __forceinline__ static void acc_zero(A& a) { a.x.hi = a.x.lo = a.y.hi = a.y.lo = 0ull; }
     __device__ __forceinline__ static void fma(A& a, V x, V y) {
-        dacc_fma(a.r0, x.re, y.re); dacc_fma(a.r1, df_neg(x.im), y.im);
-        dacc_fma(a.i0, x.re, y.im); dacc_fma(a.i1, x.im, y.re);
+        const float2 h = up2(x.h), l = up2(x.l);
+        dacc2_fma(a.x, h.x, l.x, y);
+        dacc2_fma(a.y, h.y, l.y, y);
     }
     __device__ __forceinline__ static void fms(A& a, V x, V y) {
-        dacc_fma(a.r0, df_neg(x.re), y.re); dacc_fma(a.r1, x.im, y.im);
-        dacc_fma(a.i0, df_neg(x.re), y.im); dacc_fma(a.i1, df_neg(x.im), y.re);
+        const float2 h = up2(x.h), l = up2(x.l);
+        dacc2_fma(a.x, -h.x, -l.x, y);
+        dacc2_fma(a.y, -h.y, -l.y, y);
     }
-    __device__ __forceinline__ static void add(A& a, V x) { dacc_add(a.r0, x.re); dacc_add(a.i0, x.im); }
+    __device__ __forceinline__ static void add(A& a, V x) { dacc2_add(a.x, x); }
     // a += w * x for a real w (the real part of a precision-P value)
-    __device__ __forceinline__ static void fma_real(A& a, V w, V x) { dacc_fma(a.r0, w.re, x.re); dacc_fma(a.i0, w.re, x.im); }
+    __device__ __forceinline__ static void fma_real(A& a, V w, V x) { dacc2_fma(a.x, up2(w.h).x, up2(w.l).x, x); }
     // a += w * x for a real scalar weight held exactly in a float
     typedef float S;
-    __device__ __forceinline__ static void fma_s(A& a, S w, V x) { dacc_fma_f(a.r0, w, x.re); dacc_fma_f(a.i0, w, x.im); }
-    __device__ __forceinline__ static V vadd(V a, V b) { V r; r.re = df_add(a.re, b.re); r.im = df_add(a.im, b.im); return r; }
-    // accumulator that starts from a value (chains r0, i0); get_s reads an accumulator fed
-    // only by acc_set and fma_s, which leave r1, i1 at zero, as an unnormalised pair
+    __device__ __forceinline__ static void fma_s(A& a, S w, V x) { dacc2_fma_f(a.x, w, x); }
+    __device__ __forceinline__ static V vadd(V a, V b) {
+        const df2 r = df_add2(df2{a.h, a.l}, df2{b.h, b.l});
+        V v; v.h = r.hi; v.l = r.lo; return v;
+    }
+    // accumulator that starts from a value (chain x); get_s reads an accumulator fed
+    // only by acc_set and fma_s, which leave chain y at zero, as an unnormalised pair
     // (hi + lo with |lo| small: every double-float operation here accepts that form)
-    __device__ __forceinline__ static void acc_set(A& a, V x) {
-        a.r0.hi = x.re.hi; a.r0.lo = x.re.lo; a.i0.hi = x.im.hi; a.i0.lo = x.im.lo;
-        dacc_zero(a.r1); dacc_zero(a.i1);
-    }
-    __device__ __forceinline__ static V get_s(const A& a) {
-        V v; v.re.hi = a.r0.hi; v.re.lo = a.r0.lo; v.im.hi = a.i0.hi; v.im.lo = a.i0.lo; return v;
-    }
+    __device__ __forceinline__ static void acc_set(A& a, V x) { a.x.hi = x.h; a.x.lo = x.l; a.y.hi = a.y.lo = 0ull; }
+    __device__ __forceinline__ static V get_s(const A& a) { V v; v.h = a.x.hi; v.l = a.x.lo; return v; }
     __device__ __forceinline__ static V get(const A& a) {
-        V v;
-        v.re = df_add(dacc_get(a.r0), dacc_get(a.r1));
-        v.im = df_add(dacc_get(a.i0), dacc_get(a.i1));
-        return v;
+        const df2 x = fast_two_sum2(a.x.hi, a.x.lo), y = fast_two_sum2(a.y.hi, a.y.lo);
+        const float2 h = up2(y.hi), l = up2(y.lo);
+        const df2 r = df_add2(x, df2{pk2(-h.y, h.x), pk2(-l.y, l.x)});
+        V v; v.h = r.hi; v.l = r.lo; return v;
     }
     __device__ __forceinline__ static V mul(V x, V y) {
         A a; acc_zero(a); fma(a, x, y); return get(a);
     }
-    __device__ __forceinline__ static V neg(V x) { V r; r.re = df_neg(x.re); r.im = df_neg(x.im); return r; }
+    __device__ __forceinline__ static V neg(V x) { return flip(x, -1); }
     // x for s > 0, -x otherwise, by the sign bits (integer operations only)
     __device__ __forceinline__ static V flip(V x, int s) {
-        const unsigned m = s > 0 ? 0u : 0x80000000u;
-        V r;
-        r.re.hi = __uint_as_float(__float_as_uint(x.re.hi) ^ m); r.re.lo = __uint_as_float(__float_as_uint(x.re.lo) ^ m);
-        r.im.hi = __uint_as_float(__float_as_uint(x.im.hi) ^ m); r.im.lo = __uint_as_float(__float_as_uint(x.im.lo) ^ m);
-        return r;
+        const f32x2 m = s > 0 ? 0ull : 0x8000000080000000ull;
+        V r; r.h = x.h ^ m; r.l = x.l ^ m; return r;
     }
     // Smith's complex division in double-float arithmetic
     __device__ __forceinline__ static V div(V a, V b) {
-        V r;
-        if (fabsf(b.re.hi) >= fabsf(b.im.hi)) {
-            df q = df_div(b.im, b.re);
-            df d = df_add(b.re, df_mul(b.im, q));
-            r.re = df_div(df_add(a.re, df_mul(a.im, q)), d);
-            r.im = df_div(df_add(a.im, df_neg(df_mul(a.re, q))), d);
-        } else {
-            df q = df_div(b.re, b.im);
-            df d = df_add(df_mul(b.re, q), b.im);
-            r.re = df_div(df_add(df_mul(a.re, q), a.im), d);
-            r.im = df_div(df_add(df_mul(a.im, q), df_neg(a.re)), d);
+        const df ar = cdf_re(a), ai = cdf_im(a), br = cdf_re(b), bi = cdf_im(b);
+        if (fabsf(br.hi) >= fabsf(bi.hi)) {
+            df q = df_div(bi, br);
+            df d = df_add(br, df_mul(bi, q));
+            return cdf_make(df_div(df_add(ar, df_mul(ai, q)), d), df_div(df_add(ai, df_neg(df_mul(ar, q))), d));
         }
-        return r;
+        df q = df_div(br, bi);
+        df d = df_add(df_mul(br, q), bi);
+        return cdf_make(df_div(df_add(df_mul(ar, q), ai), d), df_div(df_add(df_mul(ai, q), df_neg(ar)), d));
     }
-    __device__ __forceinline__ static float mag(V x) { return fabsf(x.re.hi) + fabsf(x.im.hi); }
-    __device__ __forceinline__ static bool is_zero(V x) { return x.re.hi == 0.f && x.im.hi == 0.f; }
+    __device__ __forceinline__ static float mag(V x) { const float2 h = up2(x.h); return fabsf(h.x) + fabsf(h.y); }
+    __device__ __forceinline__ static bool is_zero(V x) { const float2 h = up2(x.h); return h.x == 0.f && h.y == 0.f; }
     __device__ __forceinline__ static V from_cd(cd x, int e) {
-        V r; r.re = df_from_double(ldexp(x.re, e)); r.im = df_from_double(ldexp(x.im, e)); return r;
+        return cdf_make(df_from_double(ldexp(x.re, e)), df_from_double(ldexp(x.im, e)));
     }
-    __device__ __forceinline__ static cd to_cd(V x) { return cd_make(df_to_double(x.re), df_to_double(x.im)); }
+    __device__ __forceinline__ static cd to_cd(V x) { return cd_make(df_to_double(cdf_re(x)), df_to_double(cdf_im(x))); }
     __device__ __forceinline__ static bool scaled() { return true; }
     // Blocks are scaled to entries of order one; a pivot below 2^-64 is rounding residue
     // of repeated rows or columns (a zero-determinant tuple), and inverting it could
@@ -252,7 +306,7 @@ __device__ __forceinline__ V ldv(const void* base, int64_t i) {
 
 // conjugate
 __device__ __forceinline__ cd conj(cd x) { return cd_make(x.re, -x.im); }
-__device__ __forceinline__ cdf conj(cdf x) { cdf r = x; r.im = df_neg(x.im); return r; }
+__device__ __forceinline__ cdf conj(cdf x) { x.h ^= 0x8000000000000000ull; x.l ^= 0x8000000000000000ull; return x; }
 
 // ------------------------------------------------------------------ double reductions
 // Compensated double accumulator (TwoSum of each addend, errors summed separately).
