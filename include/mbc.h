@@ -149,7 +149,8 @@ typedef struct {
     int64_t minors_u, minors_d;  /* distinct minors the canonical form needs */
     int64_t tree_nodes;          /* vertices of the linearised factor tree (root included) */
     int64_t egraph_classes, egraph_nodes;     /* saturated minor e-graph size */
-    double flops_per_site;       /* algorithmic flops of this plan's algorithm, per site */
+    double flops_per_site;       /* algorithmic flops of this plan's algorithm, per site (tree: one LU
+                                    per minor; the kernels share Laplace steps between minors) */
     double direct_flops_per_site;/* the direct sweep's flops, per site (for comparison) */
     int64_t scratch_bytes_per_site; /* device scratch the algorithm uses per in-flight site */
 } mbc_plan_info;

@@ -13,6 +13,7 @@
 #include "device.cuh"
 #include "plan.hpp"
 #include "walk.hpp"
+#include "minor_levels.hpp"
 #include "tegraph.hpp"
 #include "checks.cuh"
 #include "noalloc.hpp"
@@ -42,6 +43,7 @@ struct mbc_plan {
     size_t dev_bytes = 0;
     DirectDev dd{};
     TreeDev td{};
+    int64_t tree_extra_rows = 0;  // rows of a tree plan's table below its minors
     EgraphDev ed{};
     Eg32Dev e32{};                // FP32 e-graph view (MBC_PREC_FP32 plans)
     void* dev32 = nullptr;        // its arrays (walk programs, packed words, G and pair records)
@@ -473,7 +475,7 @@ mbc_status apply_schedule(mbc_plan* P, const mbc_schedule& s) {
     return MBC_OK;
 }
 
-mbc_status upload(mbc_plan* P) {
+mbc_status upload(mbc_plan* P, const MinorLevels (&ml)[2]) {
     HostPlan& h = P->hp;
     Blob b;
     // direct
@@ -503,7 +505,46 @@ mbc_status upload(mbc_plan* P) {
         }
     size_t o_mr0 = b.add(mr[0]), o_mc0 = b.add(mc[0]), o_mr1 = b.add(mr[1]), o_mc1 = b.add(mc[1]);
     size_t o_tf = b.add(h.tree.factors), o_tc = b.add(h.tree.children), o_tco = b.add(to_val(h.tree.coefficients, pr));
-    size_t o_cn = b.add(h.tree.chunk_node), o_cl = b.add(h.tree.chunk_leaf), o_cc = b.add(h.tree.chunk_count);
+    bool real_c = h.algo == MBC_ALGO_TREE;
+    for (auto& x : h.tree.coefficients) real_c = real_c && x.imag() == 0.0 && (pr == 0 || (double)(float)x.real() == x.real());
+    std::vector<double> cd_s;
+    std::vector<float> cf_s;
+    if (real_c)
+        for (auto& x : h.tree.coefficients) {
+            if (pr == 0) cd_s.push_back(x.real());
+            else cf_s.push_back((float)x.real());
+        }
+    const size_t o_cs = pr == 0 ? b.add(cd_s) : b.add(cf_s);
+    size_t o_ml[2][7] = {};
+    for (int f = 0; f < 2; ++f)
+        for (int k = 2; k <= ml[f].n; ++k) o_ml[f][k] = b.add(ml[f].words[k]);
+    // the chunks' runs, of about equal leaf counts
+    std::vector<int64_t> run_node, run_leaf;
+    std::vector<int32_t> run_count;
+    for (size_t c = 0; c < h.tree.chunk_node.size() && h.algo == MBC_ALGO_TREE; ++c) {
+        int64_t node = h.tree.chunk_node[c], leaf = h.tree.chunk_leaf[c];
+        int64_t end = node, total = 0;
+        const int64_t n_nodes = (int64_t)h.tree.children.size(), n_leaves = (int64_t)h.tree.coefficients.size();
+        for (int32_t v = 0; v < h.tree.chunk_count[c] && end < n_nodes; ++v) {
+            const int64_t nch = h.tree.children[end];
+            if (end + 1 + nch > n_nodes || leaf + total + nch > n_leaves) break;
+            total += nch;
+            end += 1 + nch;
+        }
+        for (int r = 0; r < kTreeSplit; ++r) {
+            run_node.push_back(node);
+            run_leaf.push_back(leaf);
+            const int64_t upto = h.tree.chunk_leaf[c] + total * (r + 1) / kTreeSplit;
+            int32_t cnt = 0;
+            while (node < end && (leaf < upto || r + 1 == kTreeSplit)) {
+                leaf += h.tree.children[node];
+                node += 1 + h.tree.children[node];
+                ++cnt;
+            }
+            run_count.push_back(cnt);
+        }
+    }
+    size_t o_cn = b.add(run_node), o_cl = b.add(run_leaf), o_cc = b.add(run_count);
     // e-graph
     EgraphPlan& e = h.eg;
     struct MinorOffs { size_t child[7], row[7], pack[7], lev, col, sign, leaf; } mo[2];
@@ -612,10 +653,20 @@ mbc_status upload(mbc_plan* P) {
     td.n_minors[0] = (int64_t)h.tree.minor_rows[0].size(); td.n_minors[1] = (int64_t)h.tree.minor_rows[1].size();
     td.minor_rows[0] = at<int8_t>(dev, o_mr0); td.minor_cols[0] = at<int8_t>(dev, o_mc0);
     td.minor_rows[1] = at<int8_t>(dev, o_mr1); td.minor_cols[1] = at<int8_t>(dev, o_mc1);
+    for (int f = 0; f < 2; ++f) {
+        td.levels[f] = TreeLevelsDev();
+        td.levels[f].n = ml[f].n;
+        for (int k = 2; k <= ml[f].n; ++k) {
+            td.levels[f].words[k] = at<uint32_t>(dev, o_ml[f][k]);
+            td.levels[f].entries[k] = ml[f].rows[k];
+        }
+    }
+    td.extra_rows = P->tree_extra_rows;
     td.n_nodes = (int64_t)h.tree.factors.size();
     td.factors = at<int32_t>(dev, o_tf); td.children = at<int32_t>(dev, o_tc); td.coefficients = at<Val16>(dev, o_tco);
+    td.coef_s = real_c ? at<unsigned char>(dev, o_cs) : nullptr;
     td.n_chunks = (int)h.tree.chunk_node.size();
-    td.chunk_node = at<int64_t>(dev, o_cn); td.chunk_leaf = at<int64_t>(dev, o_cl); td.chunk_count = at<int32_t>(dev, o_cc);
+    td.run_node = at<int64_t>(dev, o_cn); td.run_leaf = at<int64_t>(dev, o_cl); td.run_count = at<int32_t>(dev, o_cc);
 
     EgraphDev& ed = P->ed;
     ed.flav_a = e.flav_a; ed.n_j = e.n_j;
@@ -665,6 +716,25 @@ mbc_status upload(mbc_plan* P) {
     return upload_f32(P);
 }
 
+// The tree's minors by shared Laplace steps where these take fewer multiply-adds than one LU per
+// minor (flops_lu leaves out the LU's pivot search and the cost of its divisions, so the line is
+// on the LU's side; the library's operators are at 0.14 to 0.57 of it).  Returns the table rows
+// below the minors.
+int64_t tree_levels(const HostPlan& h, MinorLevels (&ml)[2]) {
+    if (h.algo != MBC_ALGO_TREE) return 0;
+    const int nf[2] = {h.n_u, h.n_d};
+    int64_t extra = 0;
+    for (int f = 0; f < 2; ++f) {
+        const size_t nm = h.tree.minor_rows[f].size();
+        if (nf[f] < 2 || nm == 0) continue;
+        MinorLevels l = build_minor_levels(nf[f], h.tree.minor_rows[f], h.tree.minor_cols[f]);
+        if (8.0 * l.cfma > (double)nm * flops_lu(nf[f])) continue;
+        extra += l.extra_rows - 144;
+        ml[f] = std::move(l);
+    }
+    return ml[0].n || ml[1].n ? extra + 288 : 0;           // 288: the entries of both flavours
+}
+
 std::string signature(const HostPlan& h) {
     // identifies the plan's kernel workload for the autotune cache
     char buf[256];
@@ -691,6 +761,13 @@ mbc_status finish_plan(mbc_ctx* ctx, mbc_plan* P, mbc_plan** out) {
             i += 1 + nch;
         }
     }
+    MinorLevels ml[2];
+    try {
+        P->tree_extra_rows = tree_levels(h, ml);
+    } catch (const std::bad_alloc&) {
+        delete P;
+        return fail(ctx, MBC_OOM, "host allocation while planning the tree's minors");
+    }
     if (ctx->device < 0) {                   // host-only context: keep the host plan only
         P->signature = signature(h);
         ctx->plans.push_back(P);
@@ -700,7 +777,7 @@ mbc_status finish_plan(mbc_ctx* ctx, mbc_plan* P, mbc_plan** out) {
     }
     mbc_status st;
     try {
-        st = upload(P);
+        st = upload(P, ml);
     } catch (const std::bad_alloc&) {
         st = fail(ctx, MBC_OOM, "host allocation while uploading the plan");
     }
@@ -779,7 +856,7 @@ mbc_status run(mbc_plan* P, const void* U, const void* D, int n_sets, int T, int
     if (h.algo == MBC_ALGO_DIRECT) {
         e = launch_direct(P->dd, h.prec, u, d, g, chunk, parts, P->sched.threads, s, &c->launches);
     } else if (h.algo == MBC_ALGO_TREE) {
-        const int64_t per_site = (int64_t)(P->td.n_minors[0] + P->td.n_minors[1]) * 16;
+        const int64_t per_site = (int64_t)(P->td.n_minors[0] + P->td.n_minors[1] + P->td.extra_rows) * 16;
         int64_t wave = std::max<int64_t>(32, (int64_t)(2048LL << 20) / std::max<int64_t>(per_site, 1)) / 32 * 32;
         wave = std::min<int64_t>(wave, (n_sites + 31) / 32 * 32);
         st = ensure(c, c->scratch, (size_t)per_site * wave, s);
@@ -1034,7 +1111,7 @@ mbc_status mbc_plan_get_info(const mbc_plan* P, mbc_plan_info* info) {
     info->egraph_nodes = h.eg.A.enodes + h.eg.B.enodes;
     info->flops_per_site = h.algo == MBC_ALGO_DIRECT ? h.flops_direct : (h.algo == MBC_ALGO_TREE ? h.flops_tree : h.flops_egraph);
     info->direct_flops_per_site = h.flops_direct;
-    info->scratch_bytes_per_site = h.algo == MBC_ALGO_TREE ? (int64_t)(h.tree.minor_rows[0].size() + h.tree.minor_rows[1].size()) * 16 : 32;
+    info->scratch_bytes_per_site = h.algo == MBC_ALGO_TREE ? ((int64_t)(h.tree.minor_rows[0].size() + h.tree.minor_rows[1].size()) + P->tree_extra_rows) * 16 : 32;
     return MBC_OK;
 }
 

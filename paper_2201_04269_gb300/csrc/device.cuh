@@ -48,8 +48,16 @@ struct DirectDev {
 };
 
 // ---------------------------------------------------------------- factor tree
+// A flavour's minors by shared Laplace steps (minor_levels.hpp); n = 0: by LU.
+struct TreeLevelsDev {
+    int n;
+    const uint32_t* words[7];
+    int64_t entries[7];
+};
 struct TreeDev {
     int n_u, n_d;
+    TreeLevelsDev levels[2];
+    int64_t extra_rows;            // table rows of the levels below the minors (the entries included)
     int64_t n_minors[2];
     const int8_t* minor_rows[2];   // [m][n_f]
     const int8_t* minor_cols[2];
@@ -57,11 +65,16 @@ struct TreeDev {
     const int32_t* factors;
     const int32_t* children;
     const void* coefficients;      // precision-P values
+    const void* coef_s;            // the same as real scalars (double, or float in the mixed arithmetic)
+                                   // when every one is real and exact there, else NULL
     int n_chunks;
-    const int64_t* chunk_node;
-    const int64_t* chunk_leaf;
-    const int32_t* chunk_count;
+    // chunk c in kTreeSplit runs of whole level-1 subtrees, one per warp of its block: first node,
+    // first leaf and subtree count of run r at [c * kTreeSplit + r]
+    const int64_t* run_node;
+    const int64_t* run_leaf;
+    const int32_t* run_count;
 };
+static constexpr int kTreeSplit = 8;
 
 // ---------------------------------------------------------------- e-graph plan
 struct MinorDev {

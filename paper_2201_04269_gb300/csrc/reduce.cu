@@ -13,6 +13,25 @@ namespace mbc {
 
 __device__ __forceinline__ cd cmul(cd a, cd b) { return cd_make(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
 
+// One warp per site over its chunks (lanes take every 32nd, then a fixed shuffle tree): a
+// thread per site read its chunks one after another, strided (3He_I factor tree, 512 sites x 539
+// chunks: 640 -> 30 us).
+__global__ void chunk_reduce_kernel(Partials in, int64_t n_sites, d4* __restrict__ out) {
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= n_sites) return;
+    kacc re = {0.0, 0.0}, im = {0.0, 0.0};
+    for (int c = threadIdx.x & 31; c < in.n_chunks; c += 32) {
+        const d4 v = in.part[s * in.n_chunks + c];
+        kacc_merge(re, kacc{v.x, v.y});
+        kacc_merge(im, kacc{v.z, v.w});
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        kacc_merge(re, kacc_shfl_down(re, off));
+        kacc_merge(im, kacc_shfl_down(im, off));
+    }
+    if ((threadIdx.x & 31) == 0) out[s] = make_d4(re.hi, re.lo, im.hi, im.lo);
+}
+
 __global__ void site_reduce_kernel(Partials in, int64_t n_sites, int64_t V3, Momentum mom, cd scale, d4* site_tmp,
                                    double2* site_out) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -75,6 +94,12 @@ cudaError_t launch_reduce(Partials in, Geometry g, cd scale, double2* C, double2
                           cudaStream_t s, int64_t* launches, Momentum mom) {
     const int64_t n_sites = g.n_sites();
     const d4* sites = in.part;
+    if (in.n_chunks >= 8 && n_sites > 0) {       // (below, a thread per site is as fast)
+        chunk_reduce_kernel<<<(unsigned)((n_sites + 7) / 8), 256, 0, s>>>(in, n_sites, site_tmp);
+        ++*launches;
+        in = Partials{site_tmp, 1};
+        sites = site_tmp;
+    }
     if (in.n_chunks > 1 || site_out || mom.nonzero()) {
         const int64_t blocks = (n_sites + 255) / 256;
         if (blocks > 0) {
