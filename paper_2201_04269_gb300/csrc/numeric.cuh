@@ -204,6 +204,15 @@ struct FP64 {
         return cd_make(__longlong_as_double(__double_as_longlong(x.re) ^ m),
                        __longlong_as_double(__double_as_longlong(x.im) ^ m));
     }
+    // a d - b c.  The products are rounded the same way whatever their factors' order, so that
+    // the determinant of a block with a repeated row or column is exactly zero.
+    __device__ __forceinline__ static V det2(V a, V b, V c, V d) {
+        const V p = cd_make(__dsub_rn(__dmul_rn(a.re, d.re), __dmul_rn(a.im, d.im)),
+                            __dadd_rn(__dmul_rn(a.re, d.im), __dmul_rn(a.im, d.re)));
+        const V q = cd_make(__dsub_rn(__dmul_rn(b.re, c.re), __dmul_rn(b.im, c.im)),
+                            __dadd_rn(__dmul_rn(b.re, c.im), __dmul_rn(b.im, c.re)));
+        return cd_make(p.re - q.re, p.im - q.im);
+    }
     // Smith's complex division (R. L. Smith, 1962)
     __device__ __forceinline__ static V div(V a, V b) {
         if (fabs(b.re) >= fabs(b.im)) {
@@ -270,6 +279,10 @@ struct MIXED {
     __device__ __forceinline__ static V flip(V x, int s) {
         const f32x2 m = s > 0 ? 0ull : 0x8000000080000000ull;
         V r; r.h = x.h ^ m; r.l = x.l ^ m; return r;
+    }
+    // a d - b c (a repeated row or column leaves a residue of 2^-48 of the products)
+    __device__ __forceinline__ static V det2(V a, V b, V c, V d) {
+        A acc; acc_zero(acc); fma(acc, a, d); fms(acc, b, c); return get(acc);
     }
     // Smith's complex division in double-float arithmetic
     __device__ __forceinline__ static V div(V a, V b) {
