@@ -1493,9 +1493,12 @@ mbc_status mbc_batch(mbc_ctx* c, const mbc_work* items, int n_items, mbc_stream 
         const size_t n32 = c->batch32_host.size();
         const BatchItem32* t32 = (const BatchItem32*)c->batch32_items.p;
         const BatchItem* tdf = (const BatchItem*)((const unsigned char*)c->batch32_items.p + sizeof(BatchItem32) * n32);
+        int64_t max_v3 = 1;
+        for (const BatchItem32& it : c->batch32_host) max_v3 = std::max(max_v3, it.g.V3);
         cudaError_t e = cudaMemsetAsync(cnt + 1, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess)
-            e = launch_egraph32_batch(t32, (int)n32, c->batch32_units, c->batch32_slices, c->batch32_real,
+            e = launch_egraph32_batch(t32, (int)n32, c->batch32_units, c->batch32_slices,
+                                      max_v3, c->batch32_real,
                                       c->batch32_nj, c->batch32_cs, c->batch32_walkers, c->batch32_smem, c->sms,
                                       c->bslot.p, c->batch32_bvals, cnt + 1, (unsigned int*)c->flags.p, s,
                                       &c->launches);

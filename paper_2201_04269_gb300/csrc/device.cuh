@@ -216,10 +216,10 @@ cudaError_t launch_egraph_batch(const BatchItem* items, int n_items, int64_t n_u
 size_t egraph_kslot_bytes(const EgraphDev& d);
 // Batched FP32 launch over items (device table) sharing one cluster size, walker count
 // and shared-memory layout size (smem bytes): the FP32 kernel over every (item, site)
-// unit, then the slice guard of every item's time slices (n_slices in all).  Units to
+// unit, then the slice guard of every item's time slices (n_slices in all, of up to max_v3 sites).  Units to
 // recompute go to flag_list.  bslots: one bslot_values float2 table per cluster.
-cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t n_units, int64_t n_slices, bool real,
-                                  int nj, int cs, int walkers, int smem, int max_grid, void* bslots,
+cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t n_units, int64_t n_slices,
+                                  int64_t max_v3, bool real, int nj, int cs, int walkers, int smem, int max_grid, void* bslots,
                                   int64_t bslot_values, unsigned int* flag_count, unsigned int* flag_list,
                                   cudaStream_t s, int64_t* launches);
 // The double-float batched kernel over a device list of units (list_n: device count).

@@ -68,8 +68,13 @@ __device__ __forceinline__ void cacc_add(CAcc& a, float2 x) {
 }
 
 // Block sum of every thread's compensated complex sum and guard sum: TwoSum merges across
-// each warp in FP32, the warp results in compensated double by thread 0 (fixed order).
-// Results valid in thread 0; red holds 5 doubles per warp.
+// each warp in FP32, then the warp results in compensated double, the real parts by warp 0,
+// the imaginary parts by warp 1 and the guard by warp 2, one warp result per lane (fixed
+// order).  Results valid in thread 0; red holds 5 floats per warp and 5 doubles.  (A warp
+// instruction of the FP64 pipe, 2 lanes per cycle and SM, takes 64 cycles whatever its active
+// lanes: one thread adding 24 warps' results serially took 46k cycles a site.
+// With the staging below: proton, 512 sites, 208 -> 69 us; dinucleon I, 32768 sites, 30.6 ->
+// 22.0 ms; 3He_II-s, 27648 sites, 117.9 -> 111.1 ms.)
 __device__ __forceinline__ void block_sum_site(const CAcc& a, float guard, kacc& re, kacc& im, double& gsum,
                                                double* red) {
     float sr = a.sr, cr = a.cr, si = a.si, ci = a.ci, g = guard;
@@ -84,47 +89,101 @@ __device__ __forceinline__ void block_sum_site(const CAcc& a, float guard, kacc&
         two_sum_add(si, ci, osi);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float* rf = reinterpret_cast<float*>(red);            // [5][32]
+    double* rd = red + 80;                                // re.hi, re.lo, im.hi, im.lo, guard
     if (lane == 0) {
-        red[5 * warp + 0] = sr;
-        red[5 * warp + 1] = cr;
-        red[5 * warp + 2] = si;
-        red[5 * warp + 3] = ci;
-        red[5 * warp + 4] = g;
+        rf[warp] = sr;
+        rf[32 + warp] = cr;
+        rf[64 + warp] = si;
+        rf[96 + warp] = ci;
+        rf[128 + warp] = g;
+    }
+    __syncthreads();
+    const int part = warp;                                // (a block has at least four warps)
+    if (warp < 3) {
+        kacc k = {0.0, 0.0};
+        if (lane < nw) {
+            if (part < 2) {
+                kacc_add(k, (double)rf[64 * part + lane]);
+                kacc_add(k, (double)rf[64 * part + 32 + lane]);
+            } else {
+                k.hi = (double)rf[128 + lane];
+            }
+        }
+        for (int off = nw > 16 ? 16 : (nw > 8 ? 8 : 4); off > 0; off >>= 1) {
+            const kacc o = kacc_shfl_down(k, off);
+            if (part < 2) kacc_merge(k, o);
+            else k.hi += o.hi;
+        }
+        if (lane == 0) {
+            rd[2 * part] = k.hi;
+            if (part < 2) rd[2 * part + 1] = k.lo;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        kacc r = {0.0, 0.0}, i = {0.0, 0.0};
-        double gg = 0.0;
-        for (int w = 0; w < nw; ++w) {
-            kacc_add(r, red[5 * w + 0]);
-            kacc_add(r, red[5 * w + 1]);
-            kacc_add(i, red[5 * w + 2]);
-            kacc_add(i, red[5 * w + 3]);
-            gg += red[5 * w + 4];
-        }
-        re = r;
-        im = i;
-        gsum = gg;
+        re = kacc{rd[0], rd[1]};
+        im = kacc{rd[2], rd[3]};
+        gsum = rd[4];
     }
-    __syncthreads();
 }
 
 // Stage the site's two 12x12 blocks as FP32 values scaled by exact powers of two (the
-// largest |re|, |im| of each block in [0.5, 1)); entry (r, c) at [r * kLd + c].
+// largest |re|, |im| of each block in [0.5, 1)); entry (r, c) at [r * kLd + c].  The exponents
+// come from the high words of the values and the scaling is a change of the exponent
+// field, so that nothing but the conversion to float uses the FP64 pipe (maxima and ldexp in
+// double took 23k cycles a site); blocks whose largest entry is not well inside the normal
+// range, or with non-finite entries, take the general way.
 __device__ __forceinline__ void stage_f32(const double* __restrict__ a, const double* __restrict__ b, float2* sa,
                                           float2* sb, double* red, int& ea, int& eb) {
-    double ma = 0.0, mb = 0.0;
+    unsigned ma = 0u, mb = 0u;
+    for (int i = threadIdx.x; i < 288; i += blockDim.x) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + (i < 144 ? i : i - 144));
+        const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+        if (i < 144) ma = max(ma, m);
+        else mb = max(mb, m);
+    }
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    mb = __reduce_max_sync(0xffffffffu, mb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    unsigned* ru = reinterpret_cast<unsigned*>(red);      // [2][32]
+    if (lane == 0) {
+        ru[warp] = ma;
+        ru[32 + warp] = mb;
+    }
+    __syncthreads();
+    ma = __reduce_max_sync(0xffffffffu, lane < nw ? ru[lane] : 0u);
+    mb = __reduce_max_sync(0xffffffffu, lane < nw ? ru[32 + lane] : 0u);
+    // exponent fields of the maxima: 200..2046 (or both parts of a block zero)
+    auto plain = [](unsigned m) { return m == 0u || ((m >> 20) >= 200u && (m >> 20) < 2047u); };
+    if (plain(ma) && plain(mb)) {                         // the same for the whole block
+        ea = ma ? (int)(ma >> 20) - 1022 : 0;
+        eb = mb ? (int)(mb >> 20) - 1022 : 0;
+        for (int i = threadIdx.x; i < 288; i += blockDim.x) {
+            const int e = i < 144 ? i : i - 144;
+            const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + e);
+            const int sc = i < 144 ? ea : eb;
+            auto scaled = [sc](double x) {                // x 2^-sc (0 where that is far below the float range)
+                const int hi = __double2hiint(x), f = (hi >> 20) & 0x7ff;
+                return f - sc < 800 ? 0.f : (float)__hiloint2double(hi - (sc << 20), __double2loint(x));
+            };
+            (i < 144 ? sa : sb)[(e / 12) * kLd + e % 12] = make_float2(scaled(v.x), scaled(v.y));
+        }
+        return;
+    }
+    __syncthreads();
+    double da = 0.0, db = 0.0;
     for (int i = threadIdx.x; i < 288; i += blockDim.x) {
         const int e = i < 144 ? i : i - 144;
         const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + e);
         const double m = fmax(fabs(v.x), fabs(v.y));
-        if (i < 144) ma = fmax(ma, m);
-        else mb = fmax(mb, m);
+        if (i < 144) da = fmax(da, m);
+        else db = fmax(db, m);
     }
-    ma = block_max(ma, red);
-    mb = block_max(mb, red);
-    ea = block_exponent(ma);
-    eb = block_exponent(mb);
+    da = block_max(da, red);
+    db = block_max(db, red);
+    ea = block_exponent(da);
+    eb = block_exponent(db);
     for (int i = threadIdx.x; i < 288; i += blockDim.x) {
         const int e = i < 144 ? i : i - 144;
         const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + e);
@@ -519,7 +578,11 @@ __device__ __forceinline__ void site32(const Eg32Dev& d, const double* __restric
         store_partial(part + site, re, im, sc);
         const double cr = re.hi + re.lo, ci = im.hi + im.lo;
         const double gsum = sqrt(gs.hi + gs.lo);
-        const double est = gsum / sqrt(cr * cr + ci * ci);
+        // (without a site guard only a site whose estimate is not a number is listed: zero or
+        // non-finite sums)
+        const double est = isinf(site_guard) && cr != 0.0 && isfinite(cr) && isfinite(ci) && gsum > 0.0 && isfinite(gsum)
+                               ? 0.0
+                               : gsum / sqrt(cr * cr + ci * ci);
         // per-site guard (when per-site values are returned); a site it sends to the
         // double-float kernel has no FP32 error left for the slice guard
         const bool flag = !(est <= (double)site_guard) || !isfinite(gsum);
@@ -614,14 +677,52 @@ __global__ void __launch_bounds__(768, 1) egraph32_batch_kernel(const BatchItem3
 // or below tau leave an estimate of at most tol |C(t)| / 2 (a recomputed site carries no
 // FP32 error; tau by bisection) -- skipping sites the site guard listed already (s_x = 0).
 // C(t) here is the FP32 estimate with the momentum phase of the site sum.
+//
+// The threshold is found on the keys ceil(2^32 s_x / max s), three bits a pass, with the sums of
+// key^2 in integers (the same in any order); 40 bisection passes with FP64 divisions and
+// compensated block sums, each FP64 warp instruction 64 cycles of the pipe, took 374 us for
+// flagged slices of 64 sites and 422 us for ones of 512 (now 21 and 32 us).
 constexpr double kSliceErr = 2.5e-7;
-constexpr int kTauSteps = 40;
+constexpr int kGuardThreads = 512;
+constexpr int kGuardKeys = 40960;       // largest slice whose keys are kept in shared memory
+
+// Sum of one complex double per thread, valid in thread 0: each thread's value through shared
+// memory, warp 0 adds the real and warp 1 the imaginary parts (every 32nd value per lane, then a
+// shuffle tree), compensated.  buf: blockDim values; red: 4 doubles.  At least two warps.
+__device__ __forceinline__ void guard_sum(cd v, kacc& re, kacc& im, cd* buf, double* red) {
+    buf[threadIdx.x] = v;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        kacc k = {0.0, 0.0};
+        for (int i = lane; i < (int)blockDim.x; i += 32) kacc_add(k, warp == 0 ? buf[i].re : buf[i].im);
+        for (int off = 16; off > 0; off >>= 1) kacc_merge(k, kacc_shfl_down(k, off));
+        if (lane == 0) {
+            red[2 * warp] = k.hi;
+            red[2 * warp + 1] = k.lo;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        re = kacc{red[0], red[1]};
+        im = kacc{red[2], red[3]};
+    }
+}
+
 __device__ __forceinline__ void slice_guard_body(const d4* __restrict__ part, const double* __restrict__ scale,
                                                  int64_t st, int64_t V3, Momentum mom, double tol, int64_t unit0,
                                                  unsigned int* __restrict__ flag_count,
-                                                 unsigned int* __restrict__ flag_list, unsigned int flag_cap, double* red,
-                                                 int* s_flag, double* s_tau) {
-    double re = 0.0, im = 0.0, m = 0.0;
+                                                 unsigned int* __restrict__ flag_list, unsigned int flag_cap,
+                                                 unsigned int* keys) {
+    __shared__ cd buf[kGuardThreads];
+    __shared__ double red[4];
+    __shared__ unsigned long long wsum[7][kGuardThreads / 32], s_allow, s_max;
+    __shared__ double s_inv;
+    __shared__ int s_flag;
+    __shared__ unsigned int s_base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double re = 0.0, im = 0.0;
+    unsigned long long top = 0ull;                     // s_x >= 0: ordered as its bits
     for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) {
         const d4 v = part[st * V3 + x];
         double vr = v.x + v.y, vi = v.z + v.w;
@@ -637,74 +738,112 @@ __device__ __forceinline__ void slice_guard_body(const d4* __restrict__ part, co
         }
         re += vr;
         im += vi;
-        m = fmax(m, scale[st * V3 + x]);
+        const unsigned long long b = (unsigned long long)__double_as_longlong(scale[st * V3 + x]);
+        top = top > b ? top : b;
     }
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_down_sync(0xffffffffu, top, off);
+        top = top > o ? top : o;
+    }
+    if (lane == 0) wsum[0][warp] = top;
     kacc kr, ki;
-    block_sum(cd_make(re, im), kr, ki, red);          // valid in thread 0
-    m = block_max(m, red);
+    guard_sum(cd_make(re, im), kr, ki, buf, red);     // (its barriers order wsum too)
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < nw; ++w) top = top > wsum[0][w] ? top : wsum[0][w];
+        s_max = top;
+        s_inv = top ? 1.0 / __longlong_as_double((long long)top) : 0.0;
+    }
+    __syncthreads();
+    const double m = __longlong_as_double((long long)s_max);
+    const double inv = s_inv;
+    if (m == 0.0) return;                              // every site is listed already
+    const bool exact = isinf(inv);                     // max s_x below 2^-1022: divide
+    auto ratio = [&](int64_t x) {
+        const double sx = scale[st * V3 + x];
+        return exact ? sx / m : sx * inv;
+    };
     double q = 0.0;
-    if (m > 0.0)
-        for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) {
-            const double r = scale[st * V3 + x] / m;
-            q += r * r;
-        }
+    for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) {
+        const double r = ratio(x);
+        q += r * r;
+    }
     kacc kq, kz;
-    block_sum(cd_make(q, 0.0), kq, kz, red);
-    // the remaining sum of (s_x / m)^2 allowed after the recompute: (tol |C| / (2 kSliceErr m))^2
-    __shared__ double s_allow;
+    guard_sum(cd_make(q, 0.0), kq, kz, buf, red);
     if (threadIdx.x == 0) {
         const double cr = kr.hi + kr.lo, ci = ki.hi + ki.lo;
         const double cabs = sqrt(cr * cr + ci * ci);
         const double err = kSliceErr * m * sqrt(kq.hi + kq.lo);
-        *s_flag = m > 0.0 && !(err <= tol * cabs);
-        const double a = m > 0.0 ? tol * cabs / (2.0 * kSliceErr * m) : 0.0;
-        s_allow = isfinite(a) ? a * a : 0.0;
-        s_tau[0] = 0.0;                              // sum over s_x <= tau within the allowance
-        s_tau[1] = 1.0;                              // (every site: above it)
+        s_flag = !(err <= tol * cabs);
+        // the remaining sum of (s_x / m)^2 allowed after the recompute, (tol |C| / (2 kSliceErr m))^2,
+        // in units of 2^-32 (the sum of at most 2^31 sites stays below 2^63)
+        const double a = tol * cabs / (2.0 * kSliceErr * m);
+        s_allow = !isfinite(a) ? 0ull : (a * a >= 2147483648.0 ? 1ull << 63 : (unsigned long long)(a * a * 4294967296.0));
+        s_base = 0u;
     }
     __syncthreads();
-    if (!*s_flag) return;
-    for (int it = 0; it < kTauSteps; ++it) {
-        const double mid = 0.5 * (s_tau[0] + s_tau[1]);
-        double qb = 0.0;
+    if (!s_flag) return;
+    auto key_of = [&](int64_t x) {
+        const double r = ratio(x) * 4294967296.0;
+        return r >= 4294967295.0 ? 0xFFFFFFFFu : __double2uint_ru(r);
+    };
+    const bool kept = V3 <= kGuardKeys;
+    if (kept) {
+        for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) keys[x] = key_of(x);
+        __syncthreads();
+    }
+    // largest key threshold whose sites at or below it sum to at most the allowance
+    for (int shift = 30; shift >= 0; shift -= 3) {
+        const unsigned int base = s_base;
+        const int n = shift == 30 ? 3 : 7;             // 32 = 2 + 10 x 3 bits
+        unsigned long long sum[7] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
         for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) {
-            const double r = scale[st * V3 + x] / m;
-            if (r <= mid) qb += r * r;
+            const unsigned int k = kept ? keys[x] : key_of(x);
+            const unsigned long long k2 = ((unsigned long long)k * k + 0xFFFFFFFFull) >> 32;   // (up: 0 for k = 0 only)
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+                if (i < n && k <= base + ((unsigned int)(i + 1) << shift)) sum[i] += k2;
         }
-        kacc kb, kbz;
-        block_sum(cd_make(qb, 0.0), kb, kbz, red);
-        if (threadIdx.x == 0) {
-            if (kb.hi + kb.lo <= s_allow) s_tau[0] = mid;
-            else s_tau[1] = mid;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            for (int off = 16; off > 0; off >>= 1) sum[i] += __shfl_down_sync(0xffffffffu, sum[i], off);
+            if (lane == 0) wsum[i][warp] = sum[i];
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            unsigned long long t = 0ull;
+            if (lane < n)
+                for (int w = 0; w < nw; ++w) t += wsum[lane][w];
+            const unsigned ok = __ballot_sync(0xffffffffu, lane < n && t <= s_allow);
+            if (lane == 0) s_base = base + ((unsigned int)__popc(ok) << shift);    // (the sums ascend)
         }
         __syncthreads();
     }
-    const double tau = s_tau[0];
+    const unsigned int tau = s_base;
     for (int64_t x = threadIdx.x; x < V3; x += blockDim.x) {
-        const double sx = scale[st * V3 + x];
-        if (sx > 0.0 && sx / m > tau) {
+        if (scale[st * V3 + x] > 0.0 && (kept ? keys[x] : key_of(x)) > tau) {
             const unsigned k = atomicAdd(flag_count, 1u);
             if (!MBC_BAD(k < flag_cap, 31, k, flag_cap)) flag_list[k] = (unsigned int)(unit0 + st * V3 + x);
         }
     }
 }
 
-__global__ void slice_guard_kernel(const d4* __restrict__ part, const double* __restrict__ scale, int64_t V3,
-                                   Momentum mom, double tol, unsigned int* __restrict__ flag_count,
-                                   unsigned int* __restrict__ flag_list, unsigned int flag_cap) {
-    __shared__ double red[4 * 32];
-    __shared__ int s_flag;
-    __shared__ double s_tau[2];
-    slice_guard_body(part, scale, blockIdx.x, V3, mom, tol, 0, flag_count, flag_list, flag_cap, red, &s_flag, s_tau);
+__global__ void __launch_bounds__(kGuardThreads) slice_guard_kernel(const d4* __restrict__ part,
+                                                                    const double* __restrict__ scale, int64_t V3,
+                                                                    Momentum mom, double tol,
+                                                                    unsigned int* __restrict__ flag_count,
+                                                                    unsigned int* __restrict__ flag_list,
+                                                                    unsigned int flag_cap) {
+    extern __shared__ unsigned int guard_keys[];
+    slice_guard_body(part, scale, blockIdx.x, V3, mom, tol, 0, flag_count, flag_list, flag_cap, guard_keys);
 }
 
 // Batched slice guard: block b is slice b - slice_begin of the item whose slices contain it.
-__global__ void slice_guard_batch_kernel(const BatchItem32* __restrict__ items, int n_items,
-                                         unsigned int* __restrict__ flag_count, unsigned int* __restrict__ flag_list,
-                                         unsigned int flag_cap) {
-    __shared__ double red[4 * 32];
-    __shared__ int s_flag;
-    __shared__ double s_tau[2];
+__global__ void __launch_bounds__(kGuardThreads) slice_guard_batch_kernel(const BatchItem32* __restrict__ items,
+                                                                          int n_items,
+                                                                          unsigned int* __restrict__ flag_count,
+                                                                          unsigned int* __restrict__ flag_list,
+                                                                          unsigned int flag_cap) {
+    extern __shared__ unsigned int guard_keys[];
     int lo = 0, hi = n_items - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -713,8 +852,12 @@ __global__ void slice_guard_batch_kernel(const BatchItem32* __restrict__ items, 
     const BatchItem32& it = items[lo];
     if (std::isinf(it.slice_tol) && it.slice_tol > 0) return;
     slice_guard_body(it.part, it.scale, (int64_t)blockIdx.x - it.slice_begin, it.g.V3, Momentum(), it.slice_tol,
-                     it.unit_begin, flag_count, flag_list, flag_cap, red, &s_flag, s_tau);
+                     it.unit_begin, flag_count, flag_list, flag_cap, guard_keys);
 }
+
+// Threads and dynamic shared memory (keys) of the slice guard for slices of up to V3 sites.
+inline int guard_threads(int64_t V3) { return (int)std::min<int64_t>(kGuardThreads, std::max<int64_t>(64, (V3 + 31) / 32 * 32)); }
+inline size_t guard_smem(int64_t V3) { return V3 <= kGuardKeys ? sizeof(unsigned int) * (size_t)V3 : 0; }
 
 // Cluster launch of kern with as many clusters as can be resident at once (at most
 // `want` clusters).
@@ -790,15 +933,17 @@ cudaError_t launch_egraph32(const Eg32Dev& d, const double* U, const double* D, 
     if (e != cudaSuccess) return e;
     ++*launches;
     if (std::isinf(slice_tol) && slice_tol > 0) return cudaSuccess;      // slice guard off
-    slice_guard_kernel<<<(unsigned)((int64_t)g.n_sets * g.T), 256, 0, s>>>(part, scale, g.V3, mom, slice_tol,
-                                                                          flag_count, flag_list,
-                                                                          (unsigned int)g.n_sites());
+    const size_t gs = guard_smem(g.V3);
+    e = cudaFuncSetAttribute(slice_guard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs);
+    if (e != cudaSuccess) return e;
+    slice_guard_kernel<<<(unsigned)((int64_t)g.n_sets * g.T), guard_threads(g.V3), gs, s>>>(
+        part, scale, g.V3, mom, slice_tol, flag_count, flag_list, (unsigned int)g.n_sites());
     ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t n_units, int64_t n_slices, bool real,
-                                  int nj, int cs, int walkers, int smem, int max_grid, void* bslots,
+cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t n_units, int64_t n_slices,
+                                  int64_t max_v3, bool real, int nj, int cs, int walkers, int smem, int max_grid, void* bslots,
                                   int64_t bslot_values, unsigned int* flag_count, unsigned int* flag_list,
                                   cudaStream_t s, int64_t* launches) {
     if (n_units == 0) return cudaSuccess;
@@ -810,8 +955,12 @@ cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t
     if (e != cudaSuccess) return e;
     ++*launches;
     if (n_slices > 0) {
-        slice_guard_batch_kernel<<<(unsigned)n_slices, 256, 0, s>>>(items, n_items, flag_count, flag_list,
-                                                                     (unsigned int)n_units);
+        // (slices larger than kGuardKeys recompute their keys and need no shared memory for them)
+        const size_t gs = guard_smem(std::min<int64_t>(max_v3, kGuardKeys));
+        e = cudaFuncSetAttribute(slice_guard_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs);
+        if (e != cudaSuccess) return e;
+        slice_guard_batch_kernel<<<(unsigned)n_slices, guard_threads(max_v3), gs, s>>>(items, n_items, flag_count,
+                                                                                      flag_list, (unsigned int)n_units);
         ++*launches;
     }
     return cudaGetLastError();

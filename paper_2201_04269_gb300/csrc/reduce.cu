@@ -7,6 +7,8 @@
 // site), then over the sites of each (set, t) (one block per (set, t), a fixed
 // thread-to-site assignment and a fixed reduction tree), so the result does not depend
 // on which block computed which unit.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace mbc {
@@ -110,7 +112,9 @@ cudaError_t launch_reduce(Partials in, Geometry g, cd scale, double2* C, double2
     }
     const int64_t slices = (int64_t)g.n_sets * g.T;
     if (slices > 0) {
-        slice_reduce_kernel<<<(unsigned)slices, 256, 0, s>>>(sites, g.V3, scale, C);
+        // (a warp without sites would still pass its zeros through the FP64 pipe)
+        const int threads = (int)std::min<int64_t>(256, std::max<int64_t>(32, (g.V3 + 31) / 32 * 32));
+        slice_reduce_kernel<<<(unsigned)slices, threads, 0, s>>>(sites, g.V3, scale, C);
         ++*launches;
     }
     return cudaGetLastError();
