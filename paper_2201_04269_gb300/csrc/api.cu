@@ -710,9 +710,10 @@ mbc_status upload(mbc_plan* P, const MinorLevels (&ml)[2]) {
     // it gains more from the shorter table reads than it loses in occupancy)
     const int pk16 = (ed.A.size[ed.A.n] * ed.A.n + ed.B.size[ed.B.n] * ed.B.n + 3) / 4;
     auto resident = [](int values) { return std::min(225 * 1024 / (values * 16 + 3 * 1024), 2048 / 384); };
-    ed.stage_pk = (base + pk16) * 16 <= 200 * 1024 &&
+    // (they sit after the first 384 values, which the block sum reuses)
+    ed.stage_pk = base >= 384 && (base + pk16) * 16 <= 200 * 1024 &&
                   (h.prec == MBC_PREC_FP64 || resident(base + pk16) >= resident(base));
-    ed.smem_values = base + (ed.stage_pk ? pk16 : 0);
+    ed.smem_values = std::max(base + (ed.stage_pk ? pk16 : 0), 384);      // (the block sum takes a value per thread)
     return upload_f32(P);
 }
 

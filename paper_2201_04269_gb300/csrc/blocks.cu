@@ -362,7 +362,8 @@ template <bool SMEM>
 __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t, const cd* __restrict__ F,
                                                                    int64_t n_slices, d4* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4 * (kTreeThreads / 32)];
+    __shared__ double red[4];
+    __shared__ cd buf[kTreeThreads];
     const int64_t chunk = blockIdx.x / n_slices, slice = blockIdx.x % n_slices;
     const cd* Fs = F + slice * t.n_f;
     if (SMEM) {
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
     kacc_add(re, grp.re);
     kacc_add(im, grp.im);
     kacc ore, oim;
-    block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red);
+    block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red, buf);
     if (threadIdx.x == 0) part[slice * t.n_chunks + chunk] = make_d4(ore.hi, ore.lo, oim.hi, oim.lo);
 }
 
@@ -407,7 +408,8 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
 __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDev t, const cd* __restrict__ F,
                                                                       int64_t n_slices, d4* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4 * (kTreeThreads / 32)];
+    __shared__ double red[4];
+    __shared__ cd buf[kTreeThreads];
     __shared__ unsigned redu[64];
     const int64_t chunk = blockIdx.x / n_slices, slice = blockIdx.x % n_slices;
     const cd* Fg = F + slice * t.n_f;
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
     }
     const cd v = MIXED::to_cd(MIXED::get(tot));
     kacc ore, oim;
-    block_sum(v, ore, oim, red);
+    block_sum(v, ore, oim, red, buf);
     if (threadIdx.x == 0) {
         const double back = pow2d(max(min(t.A * e, 1000), -1000));
         part[slice * t.n_chunks + chunk] = make_d4(ore.hi * back, ore.lo * back, oim.hi * back, oim.lo * back);
@@ -464,7 +466,7 @@ __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, Block
                                                                 d4* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BlockTypeDev ty[6];
-    __shared__ double red[4 * (kThreads / 32)];
+    __shared__ double red[4];
     cd* q = reinterpret_cast<cd*>(smem_raw);
     cd* dq = q + 2 * kQ;
     cd* fs = dq + b.n_types * kDq;
@@ -501,7 +503,8 @@ __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, Block
         kacc_add(re, grp.re);
         kacc_add(im, grp.im);
         kacc ore, oim;
-        block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red);
+        // (the propagators and diquarks are done with: 720 values or more)
+        block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red, q);
         if (threadIdx.x == 0) part[site] = make_d4(ore.hi, ore.lo, oim.hi, oim.lo);
     }
 }

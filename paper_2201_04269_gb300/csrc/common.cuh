@@ -14,28 +14,29 @@ __device__ __forceinline__ kacc kacc_shfl_down(kacc v, int off) {
     return o;
 }
 
-// Deterministic compensated block sum of one complex double per thread; the result is
-// valid in thread 0.  red: shared scratch of 2 * 2 * (blockDim / 32) doubles x 2.
-__device__ __forceinline__ void block_sum(cd v, kacc& out_re, kacc& out_im, double* red) {
-    kacc re = {v.re, 0.0}, im = {v.im, 0.0};
-    for (int off = 16; off > 0; off >>= 1) {
-        kacc_merge(re, kacc_shfl_down(re, off));
-        kacc_merge(im, kacc_shfl_down(im, off));
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0) {
-        red[4 * warp + 0] = re.hi; red[4 * warp + 1] = re.lo;
-        red[4 * warp + 2] = im.hi; red[4 * warp + 3] = im.lo;
+// Deterministic compensated block sum of one complex double per thread; the result is valid
+// in thread 0.  The values go through buf (blockDim values, free after the barrier the caller
+// has passed); warp 0 adds the real parts, the last warp the imaginary parts, every 32nd value
+// per lane and then a shuffle tree: an FP64 warp instruction takes 64 cycles of the pipe
+// whatever its active lanes, so a shuffle tree in every warp costs far more.  red: 4 doubles.
+__device__ __forceinline__ void block_sum(cd v, kacc& out_re, kacc& out_im, double* red, cd* buf) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, last = (blockDim.x >> 5) - 1;
+    buf[threadIdx.x] = v;
+    __syncthreads();
+    for (int part = 0; part < 2; ++part) {
+        if (warp != (part ? last : 0)) continue;
+        kacc k = {0.0, 0.0};
+        for (int i = lane; i < (int)blockDim.x; i += 32) kacc_add(k, part ? buf[i].im : buf[i].re);
+        for (int off = 16; off > 0; off >>= 1) kacc_merge(k, kacc_shfl_down(k, off));
+        if (lane == 0) {
+            red[2 * part] = k.hi;
+            red[2 * part + 1] = k.lo;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        kacc r = {0.0, 0.0}, i = {0.0, 0.0};
-        for (int w = 0; w < nw; ++w) {
-            kacc_merge(r, kacc{red[4 * w + 0], red[4 * w + 1]});
-            kacc_merge(i, kacc{red[4 * w + 2], red[4 * w + 3]});
-        }
-        out_re = r;
-        out_im = i;
+        out_re = kacc{red[0], red[1]};
+        out_im = kacc{red[2], red[3]};
     }
     __syncthreads();
 }
@@ -51,6 +52,40 @@ __device__ __forceinline__ double block_max(double v, double* red) {
     return m;
 }
 
+// Exponents e with max |re|, |im| of each of two 12x12 blocks in [0.5, 1) after scaling by 2^-e,
+// from the high words of the values (no FP64 arithmetic): true when both maxima are well inside
+// the normal range (or zero), the same for every thread.  ru: 64 words of shared memory.
+__device__ __forceinline__ bool block_exponents(const double* __restrict__ a, const double* __restrict__ b,
+                                                unsigned* ru, int& ea, int& eb) {
+    unsigned ma = 0u, mb = 0u;
+    for (int i = threadIdx.x; i < 288; i += blockDim.x) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + (i < 144 ? i : i - 144));
+        const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+        if (i < 144) ma = max(ma, m);
+        else mb = max(mb, m);
+    }
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    mb = __reduce_max_sync(0xffffffffu, mb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) {
+        ru[warp] = ma;
+        ru[32 + warp] = mb;
+    }
+    __syncthreads();
+    ma = __reduce_max_sync(0xffffffffu, lane < nw ? ru[lane] : 0u);
+    mb = __reduce_max_sync(0xffffffffu, lane < nw ? ru[32 + lane] : 0u);
+    ea = ma ? (int)(ma >> 20) - 1022 : 0;
+    eb = mb ? (int)(mb >> 20) - 1022 : 0;
+    auto plain = [](unsigned m) { return m == 0u || ((m >> 20) >= 200u && (m >> 20) < 2047u); };
+    return plain(ma) && plain(mb);
+}
+// x 2^-e for an entry of a block whose exponent block_exponents gave, by the exponent field (0
+// where that is far below the float range)
+__device__ __forceinline__ double scaled_entry(double x, int e) {
+    const int hi = __double2hiint(x);
+    return ((hi >> 20) & 0x7ff) - e < 800 ? 0.0 : __hiloint2double(hi - (e << 20), __double2loint(x));
+}
+
 // Load two 12x12 complex double blocks (flavour matrices of one site) into shared memory
 // as precision-P values; for the mixed precision each block is first scaled by an exact
 // power of two so that its largest |re|, |im| lies in [0.5, 1); the exponents are
@@ -59,6 +94,17 @@ template <class P>
 __device__ __forceinline__ void load_pair(const double* __restrict__ a, const double* __restrict__ b,
                                           typename P::V* sa, typename P::V* sb, double* red, int& ea, int& eb) {
     // entry (r, c) goes to [r * kLd + c]
+    if (P::scaled() && block_exponents(a, b, reinterpret_cast<unsigned*>(red), ea, eb)) {
+        for (int i = threadIdx.x; i < 288; i += blockDim.x) {
+            const int e = i < 144 ? i : i - 144;
+            const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + e);
+            const int sc = i < 144 ? ea : eb;
+            (i < 144 ? sa : sb)[(e / 12) * kLd + e % 12] = P::from_scaled(cd_make(scaled_entry(v.x, sc), scaled_entry(v.y, sc)));
+        }
+        __syncthreads();
+        return;
+    }
+    if (P::scaled()) __syncthreads();           // (red is written again)
     cd* ra = reinterpret_cast<cd*>(sa);
     cd* rb = reinterpret_cast<cd*>(sb);
     double ma = 0.0, mb = 0.0;
@@ -138,7 +184,8 @@ __device__ __forceinline__ typename P::V det_gather(const typename P::V* m, cons
     return sign < 0 ? P::neg(det) : det;
 }
 
-template <class P, int LD>
+// (N: the largest n the caller needs)
+template <class P, int LD, int N = 6>
 __device__ __forceinline__ typename P::V det_n(int n, const typename P::V* m, const int8_t* rows, const int8_t* cols) {
     switch (n) {
         case 1: return m[rows[0] * LD + cols[0]];
@@ -146,10 +193,10 @@ __device__ __forceinline__ typename P::V det_n(int n, const typename P::V* m, co
         // (proton direct sweep in FP64, 512 sites: 205 -> 127 us)
         case 2: return P::det2(m[rows[0] * LD + cols[0]], m[rows[0] * LD + cols[1]], m[rows[1] * LD + cols[0]],
                                m[rows[1] * LD + cols[1]]);
-        case 3: return det_gather<P, 3, LD>(m, rows, cols);
-        case 4: return det_gather<P, 4, LD>(m, rows, cols);
-        case 5: return det_gather<P, 5, LD>(m, rows, cols);
-        case 6: return det_gather<P, 6, LD>(m, rows, cols);
+        case 3: return det_gather<P, N < 3 ? 1 : 3, LD>(m, rows, cols);
+        case 4: return det_gather<P, N < 4 ? 1 : 4, LD>(m, rows, cols);
+        case 5: return det_gather<P, N < 5 ? 1 : 5, LD>(m, rows, cols);
+        case 6: return det_gather<P, N < 6 ? 1 : 6, LD>(m, rows, cols);
         default: return P::one();   // n = 0: empty product
     }
 }

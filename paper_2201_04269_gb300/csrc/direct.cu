@@ -11,11 +11,17 @@
 // submatrices from shared memory into registers and factorises them there.  Per-thread
 // sums are combined by a deterministic compensated block reduction into one partial
 // per unit.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace mbc {
 
-template <class P>
+// N: largest minor the kernel is built for.  The registers of the 6 x 6 elimination (192 to
+// 252) left one block of 256 threads per SM for every operator; minors of up to 2 x 2
+// need a quarter of them (proton in FP64, 512 sites: 127 -> 72 us with the block sum through
+// shared memory).
+template <class P, int N>
 __global__ void __launch_bounds__(256) direct_kernel(DirectDev d, const double* __restrict__ U,
                                                      const double* __restrict__ D, Geometry g, int64_t chunk,
                                                      Partials out) {
@@ -23,6 +29,7 @@ __global__ void __launch_bounds__(256) direct_kernel(DirectDev d, const double* 
     __shared__ __align__(16) V su[kBlk];
     __shared__ __align__(16) V sd[kBlk];
     __shared__ double red[4 * 32];
+    __shared__ cd buf[256];
     const int nq = d.n_u + d.n_d;
     const int64_t n_chunks = out.n_chunks;
     const int64_t n_units = g.n_sites() * n_chunks;
@@ -76,21 +83,20 @@ __global__ void __launch_bounds__(256) direct_kernel(DirectDev d, const double* 
                     }
                 }
             }
-            int8_t ra[12], rb[12];
+            int8_t ra[2 * N], rb[2 * N];
 #pragma unroll
-            for (int i = 0; i < 12; ++i) {
+            for (int i = 0; i < 2 * N; ++i) {
                 if (i < nq) { ra[i] = ia[i]; rb[i] = ib[i]; }
             }
-            const V du = det_n<P, kLd>(d.n_u, su, ra, rb);
-            const V dd = det_n<P, kLd>(d.n_d, sd, ra + d.n_u, rb + d.n_u);
+            const V du = det_n<P, kLd, N>(d.n_u, su, ra, rb);
+            const V dd = det_n<P, kLd, N>(d.n_d, sd, ra + d.n_u, rb + d.n_u);
             const V wd = P::mul(w, du);
             P::fma(acc, wd, dd);
         }
         const cd v = P::to_cd(P::get(acc));
         kacc re, im;
-        block_sum(v, re, im, red);
+        block_sum(v, re, im, red, buf);
         if (threadIdx.x == 0) store_partial(out.part + unit, re, im, eu * d.n_u + ed * d.n_d);
-        __syncthreads();
     }
 }
 
@@ -102,8 +108,16 @@ cudaError_t launch_direct(const DirectDev& d, int prec, const double* U, const d
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = std::min<int64_t>(units, (int64_t)sms * 8);
-    if (prec == 0) direct_kernel<FP64><<<(unsigned)grid, threads, 0, s>>>(d, U, D, g, chunk, out);
-    else direct_kernel<MIXED><<<(unsigned)grid, threads, 0, s>>>(d, U, D, g, chunk, out);
+    const int n = std::max(d.n_u, d.n_d);
+#define MBC_DIRECT(P, N) direct_kernel<P, N><<<(unsigned)grid, threads, 0, s>>>(d, U, D, g, chunk, out)
+    if (prec == 0) {
+        if (n <= 2) MBC_DIRECT(FP64, 2);
+        else MBC_DIRECT(FP64, 6);
+    } else {
+        if (n <= 2) MBC_DIRECT(MIXED, 2);
+        else MBC_DIRECT(MIXED, 6);
+    }
+#undef MBC_DIRECT
     ++*launches;
     return cudaGetLastError();
 }

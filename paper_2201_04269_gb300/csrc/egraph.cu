@@ -301,9 +301,9 @@ __device__ __forceinline__ void egraph_site(const EgraphDev& d, const double* __
     // ---- site value
     const cd v = P::to_cd(P::get(acc));
     kacc re, im;
-    block_sum(v, re, im, red);
+    __syncthreads();                                   // the tables are free: their space takes the values
+    block_sum(v, re, im, red, reinterpret_cast<cd*>(smem_raw));
     if (threadIdx.x == 0) store_partial(part, re, im, ea * nA + eb * nB);
-    __syncthreads();
 }
 
 template <class P>

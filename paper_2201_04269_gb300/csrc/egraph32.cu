@@ -136,38 +136,12 @@ __device__ __forceinline__ void block_sum_site(const CAcc& a, float guard, kacc&
 // range, or with non-finite entries, take the general way.
 __device__ __forceinline__ void stage_f32(const double* __restrict__ a, const double* __restrict__ b, float2* sa,
                                           float2* sb, double* red, int& ea, int& eb) {
-    unsigned ma = 0u, mb = 0u;
-    for (int i = threadIdx.x; i < 288; i += blockDim.x) {
-        const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + (i < 144 ? i : i - 144));
-        const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
-        if (i < 144) ma = max(ma, m);
-        else mb = max(mb, m);
-    }
-    ma = __reduce_max_sync(0xffffffffu, ma);
-    mb = __reduce_max_sync(0xffffffffu, mb);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    unsigned* ru = reinterpret_cast<unsigned*>(red);      // [2][32]
-    if (lane == 0) {
-        ru[warp] = ma;
-        ru[32 + warp] = mb;
-    }
-    __syncthreads();
-    ma = __reduce_max_sync(0xffffffffu, lane < nw ? ru[lane] : 0u);
-    mb = __reduce_max_sync(0xffffffffu, lane < nw ? ru[32 + lane] : 0u);
-    // exponent fields of the maxima: 200..2046 (or both parts of a block zero)
-    auto plain = [](unsigned m) { return m == 0u || ((m >> 20) >= 200u && (m >> 20) < 2047u); };
-    if (plain(ma) && plain(mb)) {                         // the same for the whole block
-        ea = ma ? (int)(ma >> 20) - 1022 : 0;
-        eb = mb ? (int)(mb >> 20) - 1022 : 0;
+    if (block_exponents(a, b, reinterpret_cast<unsigned*>(red), ea, eb)) {
         for (int i = threadIdx.x; i < 288; i += blockDim.x) {
             const int e = i < 144 ? i : i - 144;
             const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + e);
             const int sc = i < 144 ? ea : eb;
-            auto scaled = [sc](double x) {                // x 2^-sc (0 where that is far below the float range)
-                const int hi = __double2hiint(x), f = (hi >> 20) & 0x7ff;
-                return f - sc < 800 ? 0.f : (float)__hiloint2double(hi - (sc << 20), __double2loint(x));
-            };
-            (i < 144 ? sa : sb)[(e / 12) * kLd + e % 12] = make_float2(scaled(v.x), scaled(v.y));
+            (i < 144 ? sa : sb)[(e / 12) * kLd + e % 12] = make_float2((float)scaled_entry(v.x, sc), (float)scaled_entry(v.y, sc));
         }
         return;
     }

@@ -204,14 +204,15 @@ struct FP64 {
         return cd_make(__longlong_as_double(__double_as_longlong(x.re) ^ m),
                        __longlong_as_double(__double_as_longlong(x.im) ^ m));
     }
-    // a d - b c.  The products are rounded the same way whatever their factors' order, so that
-    // the determinant of a block with a repeated row or column is exactly zero.
+    // x y - z w to about one rounding of the result (Kahan's product difference)
+    __device__ __forceinline__ static double diff(double x, double y, double z, double w) {
+        const double p = __dmul_rn(z, w);
+        return __dadd_rn(__fma_rn(x, y, -p), __fma_rn(-z, w, p));
+    }
+    // a d - b c, the real products paired so that a block with two equal rows gives exactly zero
     __device__ __forceinline__ static V det2(V a, V b, V c, V d) {
-        const V p = cd_make(__dsub_rn(__dmul_rn(a.re, d.re), __dmul_rn(a.im, d.im)),
-                            __dadd_rn(__dmul_rn(a.re, d.im), __dmul_rn(a.im, d.re)));
-        const V q = cd_make(__dsub_rn(__dmul_rn(b.re, c.re), __dmul_rn(b.im, c.im)),
-                            __dadd_rn(__dmul_rn(b.re, c.im), __dmul_rn(b.im, c.re)));
-        return cd_make(p.re - q.re, p.im - q.im);
+        return cd_make(diff(a.re, d.re, b.re, c.re) - diff(a.im, d.im, b.im, c.im),
+                       diff(a.re, d.im, b.im, c.re) + diff(a.im, d.re, b.re, c.im));
     }
     // Smith's complex division (R. L. Smith, 1962)
     __device__ __forceinline__ static V div(V a, V b) {
@@ -225,6 +226,7 @@ struct FP64 {
     __device__ __forceinline__ static double mag(V x) { return fabs(x.re) + fabs(x.im); }
     __device__ __forceinline__ static bool is_zero(V x) { return x.re == 0.0 && x.im == 0.0; }
     __device__ __forceinline__ static V from_cd(cd x, int) { return x; }
+    __device__ __forceinline__ static V from_scaled(cd x) { return x; }
     __device__ __forceinline__ static cd to_cd(V x) { return x; }
     __device__ __forceinline__ static bool scaled() { return false; }
     // smallest pivot magnitude taken as nonzero by the LU
@@ -301,6 +303,7 @@ struct MIXED {
     __device__ __forceinline__ static V from_cd(cd x, int e) {
         return cdf_make(df_from_double(ldexp(x.re, e)), df_from_double(ldexp(x.im, e)));
     }
+    __device__ __forceinline__ static V from_scaled(cd x) { return cdf_make(df_from_double(x.re), df_from_double(x.im)); }
     __device__ __forceinline__ static cd to_cd(V x) { return cd_make(df_to_double(cdf_re(x)), df_to_double(cdf_im(x))); }
     __device__ __forceinline__ static bool scaled() { return true; }
     // Blocks are scaled to entries of order one; a pivot below 2^-64 is rounding residue
