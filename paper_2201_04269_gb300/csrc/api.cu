@@ -384,6 +384,8 @@ std::string add_f32(const HostPlan& h, const F32Shape& shape, Eg32Dev& v, Blob& 
     v.leafbuf_vals = LB * leaf_size;
     v.pk_words = pk_words;
     v.smem_bytes = f32_smem(W, LB, pk_words, stack_vals, leaf_size);
+    // two blocks per SM for minors up to 2 x 2 with real weights (egraph32.cu)
+    v.blocks = real && std::max(e.A.n, e.B.n) <= 2 && cs == 1 && nj <= 2 && v.smem_bytes <= 110 * 1024 ? 2 : 1;
     v.n_cols_a = (int)e.A.cols.size();
     v.n_terms = (int64_t)t4.size();
     v.n_sell = (int64_t)sc.size();
@@ -867,7 +869,7 @@ mbc_status run(mbc_plan* P, const void* U, const void* D, int n_sets, int T, int
     } else if (h.prec == MBC_PREC_FP32) {
         // FP32 pass (one block per SM, a B table per block), then the double-float
         // kernel over the sites whose error estimate exceeded the guard
-        const int grid32 = c->sms;
+        const int grid32 = c->sms * P->e32.blocks;
         const int grid_df = (int)std::min<int64_t>(n_sites, (int64_t)c->sms * P->sched_df.blocks_per_sm);
         st = ensure(c, c->bslot, sizeof(float2) * (size_t)P->e32.n_cols_b * P->e32.n_rows_b * (grid32 / P->e32.cs), s);
         if (st == MBC_OK) st = ensure(c, c->flags, sizeof(unsigned int) * (size_t)n_sites, s);

@@ -140,6 +140,7 @@ struct Eg32Dev {
     int flav_a, n_j, real_w;
     int walkers, lb;                 // walkers per block, leaf batch size of the A flavour
     int cs;                          // blocks per site (a thread-block cluster when > 1)
+    int blocks;                      // resident blocks per SM of the single-plan kernel
     int n_rows_b, n_cols_b;          // the B table of a site is n_cols_b x n_rows_b
     int stack_vals;                  // float2 values of a walker's table stack
     int leafbuf_vals;                // lb x size_A[n_A]

@@ -239,28 +239,31 @@ __device__ __forceinline__ void lap_leaves(const float2* M, const uint32_t* pk, 
     }
 }
 
+// (KM: the largest level of the plans the kernel is built for)
+template <int KM>
 __device__ __forceinline__ void lap_node_k(int k, const float2* M, const uint32_t* pk, int n, int col, int sign,
                                            const float2* parent, float2* dest, int wt, int n_parent) {
     switch (k) {
         case 1: lap_node<1>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
         case 2: lap_node<2>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
-        case 3: lap_node<3>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
-        case 4: lap_node<4>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
-        case 5: lap_node<5>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
-        default: lap_node<6>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
+        case 3: lap_node<KM < 3 ? 1 : 3>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
+        case 4: lap_node<KM < 4 ? 1 : 4>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
+        case 5: lap_node<KM < 5 ? 1 : 5>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
+        default: lap_node<KM < 6 ? 1 : 6>(M, pk, n, col, sign, parent, dest, wt, n_parent); break;
     }
 }
 
+template <int KM>
 __device__ __forceinline__ void lap_leaves_k(int k, const float2* M, const uint32_t* pk, int n, const WalkLeaf* lv,
                                              int nleaf, const float2* parent, float2* out, bool to_cols, int wt,
                                              int n_parent, int64_t out_bound, const int32_t* opos) {
     switch (k) {
         case 1: lap_leaves<1>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
         case 2: lap_leaves<2>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
-        case 3: lap_leaves<3>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
-        case 4: lap_leaves<4>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
-        case 5: lap_leaves<5>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
-        default: lap_leaves<6>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
+        case 3: lap_leaves<KM < 3 ? 1 : 3>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
+        case 4: lap_leaves<KM < 4 ? 1 : 4>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
+        case 5: lap_leaves<KM < 5 ? 1 : 5>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
+        default: lap_leaves<KM < 6 ? 1 : 6>(M, pk, n, lv, nleaf, parent, out, to_cols, wt, n_parent, out_bound, opos); break;
     }
 }
 
@@ -405,7 +408,7 @@ __device__ __forceinline__ void leaf_stage(const Eg32Dev& d, const WalkLeaf* lv,
 
 // Run one flavour's walker program: B (to_cols: leaf tables to the block's B table) or
 // A (leaf tables to the walker's batch buffer, then the leaf stage).
-template <bool REAL, int NJ>
+template <bool REAL, int NJ, int KM>
 __device__ __forceinline__ void walk(const Eg32Dev& d, const WalkDev& f, bool is_a, const float2* M,
                                      const uint32_t* spk, float2* stack, float2* leafbuf, float2* bt, CAcc& acc,
                                      float& guard, int gw, int w, int wt) {
@@ -422,14 +425,14 @@ __device__ __forceinline__ void walk(const Eg32Dev& d, const WalkDev& f, bool is
         }
         if (st.level > 0) {
             const int k = st.level;
-            lap_node_k(k, M, spk + f.pk_off[k], f.size[k], st.col, st.sign, stack + f.off[k - 1], stack + f.off[k], wt,
+            lap_node_k<KM>(k, M, spk + f.pk_off[k], f.size[k], st.col, st.sign, stack + f.off[k - 1], stack + f.off[k], wt,
                        f.size[k - 1]);
             walker_sync(w);
         }
         if (st.nleaf > 0) {
             if (st.level == 0) walker_sync(w);     // the previous batch may still be read
             const WalkLeaf* lv = f.leaves + st.leaf0;
-            lap_leaves_k(n, M, spk + f.pk_off[n], f.size[n], lv, st.nleaf, stack + f.off[n - 1],
+            lap_leaves_k<KM>(n, M, spk + f.pk_off[n], f.size[n], lv, st.nleaf, stack + f.off[n - 1],
                          is_a ? leafbuf : bt, !is_a, wt, f.size[n - 1],
                          is_a ? (int64_t)d.leafbuf_vals : (int64_t)d.n_cols_b * d.n_rows_b, d.b_pos);
             walker_sync(w);
@@ -494,7 +497,7 @@ __device__ __forceinline__ void site32_stage_plan(const Eg32Dev& d, const Site32
 // its partial sums to block 0 of the cluster, which combines them in rank order
 // (deterministic).  Block 0 writes the site's partial and error scale and, when the
 // per-site estimate exceeds site_guard, appends `unit` to the recompute list.
-template <bool REAL, int NJ>
+template <bool REAL, int NJ, int KM>
 __device__ __forceinline__ void site32(const Eg32Dev& d, const double* __restrict__ U, const double* __restrict__ D,
                                        int64_t site, int64_t unit, d4* __restrict__ part, double* __restrict__ scale_out,
                                        float2* __restrict__ bt, const Site32Smem& m, int rank, int cs,
@@ -517,11 +520,11 @@ __device__ __forceinline__ void site32(const Eg32Dev& d, const double* __restric
     if (nB == 0) {
         if (threadIdx.x == 0 && rank == 0) bt[0] = make_float2(1.f, 0.f);
     } else if (active) {
-        walk<REAL, NJ>(d, d.B, false, m.sB, m.spk, m.stack, m.leafbuf, bt, acc, guard, gw, w, wt);
+        walk<REAL, NJ, KM>(d, d.B, false, m.sB, m.spk, m.stack, m.leafbuf, bt, acc, guard, gw, w, wt);
     }
     __syncthreads();                                   // the B table is complete
     if (cs > 1) cluster_sync_all();
-    if (active) walk<REAL, NJ>(d, d.A, true, m.sA, m.spk, m.stack, m.leafbuf, bt, acc, guard, gw, w, wt);
+    if (active) walk<REAL, NJ, KM>(d, d.A, true, m.sA, m.spk, m.stack, m.leafbuf, bt, acc, guard, gw, w, wt);
     // site value: compensated block sums of the parts and of |part|^2
     kacc re = {0.0, 0.0}, im = {0.0, 0.0}, gs = {0.0, 0.0};
     block_sum_site(acc, guard, re, im, gs.hi, m.red);
@@ -568,9 +571,14 @@ __device__ __forceinline__ void site32(const Eg32Dev& d, const double* __restric
     }
 }
 
-// One plan: sites assigned round robin to the grid's clusters.
-template <bool REAL, int NJ>
-__global__ void __launch_bounds__(768, 1) egraph32_kernel(Eg32Dev d, const double* __restrict__ U,
+// One plan: sites assigned round robin to the grid's clusters.  KM = 2 (plans of minors up to 2 x 2,
+// d.blocks == 2): two blocks per SM at 40 registers.  Such a site is mostly latency (staging,
+// a few short batches, the block sum), which a second site in flight fills: proton, guards off,
+// 512 sites 81 -> 62 us, 32768 sites 3.24 -> 2.30 ms.  Dinucleon I (3 x 3) spills at 40 registers
+// and has two B tables in flight per SM near the size of the L2: 10.2 -> 11.6 ms for 16384 sites, so it
+// keeps one block.
+template <bool REAL, int NJ, int KM>
+__global__ void __launch_bounds__(768, KM <= 2 ? 2 : 1) egraph32_kernel(const __grid_constant__ Eg32Dev d, const double* __restrict__ U,
                                                           const double* __restrict__ D, Geometry g,
                                                           d4* __restrict__ part, float2* __restrict__ bslots,
                                                           unsigned int* __restrict__ flag_count,
@@ -587,7 +595,7 @@ __global__ void __launch_bounds__(768, 1) egraph32_kernel(Eg32Dev d, const doubl
     site32_stage_plan(d, m);
     const int64_t n_units = g.n_sites();
     for (int64_t site = cid; site < n_units; site += ncl)
-        site32<REAL, NJ>(d, U, D, site, site, part, scale_out, bt, m, rank, d.cs, site_guard, flag_count, flag_list,
+        site32<REAL, NJ, KM>(d, U, D, site, site, part, scale_out, bt, m, rank, d.cs, site_guard, flag_count, flag_list,
                          flag_cap);
 }
 
@@ -634,7 +642,7 @@ __global__ void __launch_bounds__(768, 1) egraph32_batch_kernel(const BatchItem3
         }
         const BatchItem32& item = items[it];
         const Site32Smem m = site32_smem(sd, smem_raw, red, xpart);
-        site32<REAL, NJ>(sd, item.U, item.D, unit - item.unit_begin, unit, item.part, item.scale, bt, m, rank, cs,
+        site32<REAL, NJ, 6>(sd, item.U, item.D, unit - item.unit_begin, unit, item.part, item.scale, bt, m, rank, cs,
                          item.site_guard, flag_count, flag_list, flag_cap);
     }
 }
@@ -867,11 +875,11 @@ cudaError_t launch_clusters(K kern, int cs, int walkers, int smem, int64_t want,
     return cudaGetLastError();
 }
 
-template <bool REAL, int NJ>
+template <bool REAL, int NJ, int KM = 6>
 cudaError_t launch_t(const Eg32Dev& d, const double* U, const double* D, Geometry g, d4* part, int max_grid,
                      void* bslots, unsigned int* flag_count, unsigned int* flag_list, float site_guard,
                      double* scale_out, cudaStream_t s) {
-    return launch_clusters(egraph32_kernel<REAL, NJ>, d.cs, d.walkers, d.smem_bytes, g.n_sites(), max_grid, s, d, U,
+    return launch_clusters(egraph32_kernel<REAL, NJ, KM>, d.cs, d.walkers, d.smem_bytes, g.n_sites(), max_grid, s, d, U,
                            D, g, part, (float2*)bslots, flag_count, flag_list, site_guard, scale_out,
                            (unsigned int)g.n_sites());
 }
@@ -893,8 +901,8 @@ cudaError_t launch_egraph32(const Eg32Dev& d, const double* U, const double* D, 
     cudaError_t e;
 #define MBC_E32_ARGS d, U, D, g, part, max_grid, bslots, flag_count, flag_list, site_guard, scale, s
     switch (d.n_j * 2 + (d.real_w ? 1 : 0)) {
-        case 3: e = launch_t<true, 1>(MBC_E32_ARGS); break;
-        case 5: e = launch_t<true, 2>(MBC_E32_ARGS); break;
+        case 3: e = d.blocks == 2 ? launch_t<true, 1, 2>(MBC_E32_ARGS) : launch_t<true, 1>(MBC_E32_ARGS); break;
+        case 5: e = d.blocks == 2 ? launch_t<true, 2, 2>(MBC_E32_ARGS) : launch_t<true, 2>(MBC_E32_ARGS); break;
         case 7: e = launch_t<true, 3>(MBC_E32_ARGS); break;
         case 9: e = launch_t<true, 4>(MBC_E32_ARGS); break;
         case 2: e = launch_t<false, 1>(MBC_E32_ARGS); break;
