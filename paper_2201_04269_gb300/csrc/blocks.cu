@@ -13,6 +13,9 @@
 // their running sums over the block's sites in shared memory, so the kernel reads 4.6 KB
 // per site and writes one partial block per tile of sites.  Arithmetic: complex double;
 // the kernel is bound by the FP64 pipe.
+#include <algorithm>
+#include <cstdint>
+
 #include "blocks.cuh"
 #include "common.cuh"
 
@@ -56,7 +59,10 @@ __device__ __forceinline__ void load_types(const BlockDev& b, BlockTypeDev* ty) 
     if (threadIdx.x < b.n_types) ty[threadIdx.x] = b.t[threadIdx.x];
 }
 
-__device__ __forceinline__ void diquarks(int n_types, const BlockTypeDev* types, const cd* q, cd* dq) {
+// mom: times the phase ph (a block is linear in its diquark, so the projection's phase is taken
+// here, on 432 values a type, not on its several thousand entries)
+__device__ __forceinline__ void diquarks(int n_types, const BlockTypeDev* types, const cd* q, cd* dq, bool mom = false,
+                                         cd ph = cd_make(1.0, 0.0)) {
     for (int e = threadIdx.x; e < n_types * kDq; e += blockDim.x) {
         const int t = e / kDq, r = e - t * kDq;
         const int c = r / 144, s = (r / 12) % 12, s2 = r % 12;
@@ -73,7 +79,7 @@ __device__ __forceinline__ void diquarks(int n_types, const BlockTypeDev* types,
             x.im -= y.im;
             cfma(acc, cd_make(ty.g_re[k], ty.g_im[k]), x);
         }
-        dq[e] = acc;
+        dq[e] = mom ? cmul(acc, ph) : acc;
     }
 }
 
@@ -123,6 +129,7 @@ __global__ void __launch_bounds__(kThreads) block_project_kernel(BlockDev b, con
                                                                   int n_fc, cd* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BlockTypeDev ty[6];
+    __shared__ cd ph_s;
     cd* q = reinterpret_cast<cd*>(smem_raw);
     cd* dq = q + 2 * kQ;
     cd* acc = dq + b.n_types * kDq;
@@ -139,28 +146,23 @@ __global__ void __launch_bounds__(kThreads) block_project_kernel(BlockDev b, con
     for (int64_t x = x0; x < x1; ++x) {
         __syncthreads();
         stage_site(U, D, slice * V3 + x, q);
-        __syncthreads();
-        diquarks(b.n_types, ty, q, dq);
-        __syncthreads();
         cd ph = cd_make(1.0, 0.0);
         if (mom) {
             const int64_t cx = x % L, cy = (x / L) % L, cz = x / ((int64_t)L * L);
             int64_t k = ((int64_t)px * cx + (int64_t)py * cy + (int64_t)pz * cz) % L;
             if (k < 0) k += L;
-            double sn, cs;
-            sincospi(-2.0 * (double)k / (double)L, &sn, &cs);
-            ph = cd_make(cs, sn);
-        }
-        if (mom) {
-            for (int f = threadIdx.x; f < nf; f += blockDim.x) {
-                const cd v = cmul(block_entry(ty, entry_code(b, f0 + f), q, dq), ph);
-                acc[f].re += v.re;
-                acc[f].im += v.im;
+            if (threadIdx.x == 0) {                  // (FP64 arithmetic: by one warp, not by all)
+                double sn, cs;
+                sincospi(-2.0 * (double)k / (double)L, &sn, &cs);
+                ph_s = cd_make(cs, sn);
             }
-        } else {
-            // the running sum is the first addend of the entry's multiply-add chain
-            for (int f = threadIdx.x; f < nf; f += blockDim.x) acc[f] = block_entry(ty, entry_code(b, f0 + f), q, dq, acc[f]);
         }
+        __syncthreads();
+        if (mom) ph = ph_s;
+        diquarks(b.n_types, ty, q, dq, mom, ph);
+        __syncthreads();
+        // the running sum is the first addend of the entry's multiply-add chain
+        for (int f = threadIdx.x; f < nf; f += blockDim.x) acc[f] = block_entry(ty, entry_code(b, f0 + f), q, dq, acc[f]);
     }
     cd* o = part + (slice * tiles + tile) * (int64_t)b.n_f + f0;
     for (int f = threadIdx.x; f < nf; f += blockDim.x) o[f] = acc[f];
@@ -216,7 +218,9 @@ __device__ __forceinline__ void stage_site_df(const double* __restrict__ U, cons
     }
 }
 
-__device__ __forceinline__ void diquarks_df(int n_types, const BlockTypeDev* types, const cdf* q, cdf* dq) {
+// sc0, sc1: the site's power of two for blocks with q1 = u, d; mom: times the phase ph too
+__device__ __forceinline__ void diquarks_df(int n_types, const BlockTypeDev* types, const cdf* q, cdf* dq, float sc0,
+                                            float sc1, bool mom, const cdf& ph) {
     for (int e = threadIdx.x; e < n_types * kDq; e += blockDim.x) {
         const int t = e / kDq, r = e - t * kDq;
         const int c = r / 144, s = (r / 12) % 12, s2 = r % 12;
@@ -237,7 +241,9 @@ __device__ __forceinline__ void diquarks_df(int n_types, const BlockTypeDev* typ
                 MIXED::fma(acc, q1[(rb + b0) * 12 + s], q2[(rg + a0) * 12 + s2]);
             }
         }
-        dq[e] = MIXED::get(acc);
+        cdf v = MIXED::get(acc);
+        if (mom) v = MIXED::mul(v, ph);
+        dq[e] = cdf_scale(v, ty.q1 ? sc1 : sc0);
     }
 }
 
@@ -320,17 +326,14 @@ __global__ void __launch_bounds__(kThreads) block_project_df_kernel(BlockDev b, 
             ph_s = cdf_make(df_from_double(cs), df_from_double(sn));
         }
         __syncthreads();
-        diquarks_df(b.n_types, ty, q, dq);
+        // (a block is linear in its diquark: the site's scale and phase are taken there, on 432 values
+        // a type: 3He_II-s with momentum, 16384 sites, 3.3 -> 2.44 ms with the tile counts of
+        // project_shape.  Starting the entries' chains from the running sums would save another 6 %, and
+        // doubled the error.)
+        diquarks_df(b.n_types, ty, q, dq, pow2f_le0(2 * eU + eD - eref[0]), pow2f_le0(2 * eD + eU - eref[1]), mom, ph_s);
         __syncthreads();
-        const float sc0 = pow2f_le0(2 * eU + eD - eref[0]), sc1 = pow2f_le0(2 * eD + eU - eref[1]);
-        const cdf ph = ph_s;
-        for (int f = threadIdx.x; f < nf; f += blockDim.x) {
-            const uint32_t code = entry_code(b, f0 + f);
-            cdf v = block_entry_df(ty, code, q, dq);
-            if (mom) v = MIXED::mul(v, ph);
-            const float sc = ty[code >> 16].q1 ? sc1 : sc0;
-            acc[f] = MIXED::vadd(acc[f], cdf_scale(v, sc));
-        }
+        for (int f = threadIdx.x; f < nf; f += blockDim.x)
+            acc[f] = MIXED::vadd(acc[f], block_entry_df(ty, entry_code(b, f0 + f), q, dq));
     }
     cd* o = part + (slice * tiles + tile) * (int64_t)b.n_f + f0;
     const double s0 = pow2d(max(min(eref[0], 1000), -1000)), s1 = pow2d(max(min(eref[1], 1000), -1000));
@@ -341,30 +344,74 @@ __global__ void __launch_bounds__(kThreads) block_project_df_kernel(BlockDev b, 
     }
 }
 
-// F[slice][f] = sum over tiles in order (compensated)
-__global__ void block_tile_reduce_kernel(const cd* __restrict__ part, int64_t n_slices, int tiles, int n_f,
-                                         cd* __restrict__ F) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_slices * n_f) return;
-    const int64_t slice = i / n_f, f = i % n_f;
+// F[slice][f] = sum over tiles (compensated): a block takes 32 entries, its warps every 8th tile each,
+// combined in order.  (One thread per entry added its tiles one after another, each addition 12
+// FP64 instructions of 64 cycles: 138 us for 9288 entries x 128 tiles.  Four such slices now take
+// 146 us, two thirds of that at the rate of the FP64 pipe.)
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps) block_tile_reduce_kernel(const cd* __restrict__ part,
+                                                                               int64_t n_slices, int tiles, int n_f,
+                                                                               cd* __restrict__ F) {
+    __shared__ d4 sum[kReduceWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    const bool live = i < n_slices * n_f;
+    const int64_t slice = live ? i / n_f : 0, f = live ? i % n_f : 0;
     kacc re = {0.0, 0.0}, im = {0.0, 0.0};
-    for (int t = 0; t < tiles; ++t) {
+    for (int t = warp; t < tiles; t += kReduceWarps) {
         const cd v = part[(slice * tiles + t) * n_f + f];
         kacc_add(re, v.re);
         kacc_add(im, v.im);
     }
+    sum[warp][lane] = make_d4(re.hi, re.lo, im.hi, im.lo);
+    __syncthreads();
+    if (warp != 0 || !live) return;
+    for (int w = 1; w < kReduceWarps; ++w) {
+        const d4 v = sum[w][lane];
+        kacc_merge(re, kacc{v.x, v.y});
+        kacc_merge(im, kacc{v.z, v.w});
+    }
     F[i] = cd_make(re.hi + re.lo, im.hi + im.lo);
 }
 
-// unit = (chunk, slice), chunk-major so that the blocks working on one chunk of the tree
-// run together and share its arrays in L2
-template <bool SMEM>
+// One unit of the block factor tree in complex double: the product of its path's factors times
+// the weighted sum of its leaves, added to grp.  Real weights (all of the library's) take
+// half the multiply-adds and one 8-byte record a leaf: dinucleon I at the local sink, 4096 sites,
+// 3.12 -> 2.36 ms, bound by the FP64 pipe.
+template <bool REAL>
+__device__ __forceinline__ void tree_unit(const BlockTreeDev& t, int64_t u, int np, const cd* Fs, cd& grp) {
+    cd pre = np ? Fs[__ldg(t.unit_pre + u * np)] : cd_make(1.0, 0.0);
+    for (int k = 1; k < np; ++k) pre = cmul(pre, Fs[__ldg(t.unit_pre + u * np + k)]);
+    cd s = cd_make(0.0, 0.0);
+    const int32_t l1 = __ldg(t.unit_leaf + u + 1);
+    for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
+        if (REAL) {
+            const uint2 r = __ldg(t.leaf_rd + l);
+            const double w = __hiloint2double((int)r.y, 0);
+            const cd f = Fs[r.x];
+            s.re = fma(w, f.re, s.re);
+            s.im = fma(w, f.im, s.im);
+        } else {
+            const double2 w = __ldg(t.leaf_wd + l);
+            cfma(s, cd_make(w.x, w.y), Fs[__ldg(t.leaf_f + l)]);
+        }
+    }
+    cfma(grp, pre, s);
+}
+
+// Block (g, slice) walks chunks g, g + groups, ... of the tree for one slice, g-major so that the
+// blocks working on one chunk run together and share its arrays in L2.  The slice's
+// projected blocks are loaded (double-float: scaled and split, FP64 arithmetic worth a chunk's
+// walk) once for all of them (launch_block_tree chooses the groups).  3He_II-s double-float, 4 slices: 680 ->
+// 503 us against one block per chunk.
+template <bool SMEM, bool REAL>
 __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t, const cd* __restrict__ F,
-                                                                   int64_t n_slices, d4* __restrict__ part) {
+                                                                   int64_t n_slices, int groups,
+                                                                   d4* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[4];
     __shared__ cd buf[kTreeThreads];
-    const int64_t chunk = blockIdx.x / n_slices, slice = blockIdx.x % n_slices;
+    const int64_t slice = blockIdx.x % n_slices;
     const cd* Fs = F + slice * t.n_f;
     if (SMEM) {
         cd* fs = reinterpret_cast<cd*>(smem_raw);
@@ -373,45 +420,41 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
         Fs = fs;
     }
     const int np = t.A - 1;
-    kacc re = {0.0, 0.0}, im = {0.0, 0.0};
-    // units are added in groups of four in plain double, each group's sum compensated
-    cd grp = cd_make(0.0, 0.0);
-    int in_grp = 0;
-    for (int64_t u = t.chunk_unit[chunk] + threadIdx.x; u < t.chunk_unit[chunk + 1]; u += blockDim.x) {
-        cd pre = cd_make(1.0, 0.0);
-        for (int k = 0; k < np; ++k) pre = cmul(pre, Fs[__ldg(t.unit_pre + u * np + k)]);
-        cd s = cd_make(0.0, 0.0);
-        const int32_t l1 = __ldg(t.unit_leaf + u + 1);
-        for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
-            const double2 w = __ldg(t.leaf_wd + l);
-            cfma(s, cd_make(w.x, w.y), Fs[__ldg(t.leaf_f + l)]);
+    for (int chunk = (int)(blockIdx.x / n_slices); chunk < t.n_chunks; chunk += groups) {
+        kacc re = {0.0, 0.0}, im = {0.0, 0.0};
+        // units are added in groups of four in plain double, each group's sum compensated
+        cd grp = cd_make(0.0, 0.0);
+        int in_grp = 0;
+        for (int64_t u = t.chunk_unit[chunk] + threadIdx.x; u < t.chunk_unit[chunk + 1]; u += blockDim.x) {
+            tree_unit<REAL>(t, u, np, Fs, grp);
+            if (++in_grp == 4) {
+                kacc_add(re, grp.re);
+                kacc_add(im, grp.im);
+                grp = cd_make(0.0, 0.0);
+                in_grp = 0;
+            }
         }
-        cfma(grp, pre, s);
-        if (++in_grp == 4) {
-            kacc_add(re, grp.re);
-            kacc_add(im, grp.im);
-            grp = cd_make(0.0, 0.0);
-            in_grp = 0;
-        }
+        kacc_add(re, grp.re);
+        kacc_add(im, grp.im);
+        kacc ore, oim;
+        block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red, buf);
+        if (threadIdx.x == 0) part[slice * t.n_chunks + chunk] = make_d4(ore.hi, ore.lo, oim.hi, oim.lo);
     }
-    kacc_add(re, grp.re);
-    kacc_add(im, grp.im);
-    kacc ore, oim;
-    block_sum(cd_make(re.hi + re.lo, im.hi + im.lo), ore, oim, red, buf);
-    if (threadIdx.x == 0) part[slice * t.n_chunks + chunk] = make_d4(ore.hi, ore.lo, oim.hi, oim.lo);
 }
 
 // The same walk in double-float arithmetic: the slice's projected blocks are scaled by an
 // exact power of two 2^-e (e from the largest |re|, |im| among them) into (hi, lo) float
 // pairs in shared memory; a term of A factors then carries 2^(A e), restored in double
 // on the block's partial sum.
+template <bool REAL>
 __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDev t, const cd* __restrict__ F,
-                                                                      int64_t n_slices, d4* __restrict__ part) {
+                                                                      int64_t n_slices, int groups,
+                                                                      d4* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[4];
     __shared__ cd buf[kTreeThreads];
     __shared__ unsigned redu[64];
-    const int64_t chunk = blockIdx.x / n_slices, slice = blockIdx.x % n_slices;
+    const int64_t slice = blockIdx.x % n_slices;
     const cd* Fg = F + slice * t.n_f;
     cdf* fs = reinterpret_cast<cdf*>(smem_raw);
     unsigned m = 0u, m2 = 0u;
@@ -428,29 +471,36 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
     }
     __syncthreads();
     const int np = t.A - 1;
-    MIXED::A tot;
-    MIXED::acc_zero(tot);
-    for (int64_t u = t.chunk_unit[chunk] + threadIdx.x; u < t.chunk_unit[chunk + 1]; u += blockDim.x) {
-        cdf pre = MIXED::one();
-        for (int k = 0; k < np; ++k) pre = MIXED::mul(pre, fs[__ldg(t.unit_pre + u * np + k)]);
-        MIXED::A a;
-        MIXED::acc_zero(a);
-        const int32_t l1 = __ldg(t.unit_leaf + u + 1);
-        for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
-            const float2 w = __ldg(t.leaf_w + l);
-            const cdf f = fs[__ldg(t.leaf_f + l)];
-            // (w.x + i w.y) f with float weights (exact products by error-free transformation)
-            dacc2_fma_f(a.x, w.x, f);
-            dacc2_fma_f(a.y, w.y, f);
+    for (int chunk = (int)(blockIdx.x / n_slices); chunk < t.n_chunks; chunk += groups) {
+        MIXED::A tot;
+        MIXED::acc_zero(tot);
+        for (int64_t u = t.chunk_unit[chunk] + threadIdx.x; u < t.chunk_unit[chunk + 1]; u += blockDim.x) {
+            cdf pre = np ? fs[__ldg(t.unit_pre + u * np)] : MIXED::one();
+            for (int k = 1; k < np; ++k) pre = MIXED::mul(pre, fs[__ldg(t.unit_pre + u * np + k)]);
+            MIXED::A a;
+            MIXED::acc_zero(a);
+            const int32_t l1 = __ldg(t.unit_leaf + u + 1);
+            for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
+                if (REAL) {
+                    const uint2 r = __ldg(t.leaf_rf + l);
+                    dacc2_fma_f(a.x, __uint_as_float(r.y), fs[r.x]);
+                    continue;
+                }
+                const float2 w = __ldg(t.leaf_w + l);
+                const cdf f = fs[__ldg(t.leaf_f + l)];
+                // (w.x + i w.y) f with float weights (exact products by error-free transformation)
+                dacc2_fma_f(a.x, w.x, f);
+                dacc2_fma_f(a.y, w.y, f);
+            }
+            MIXED::fma(tot, pre, REAL ? MIXED::get_s(a) : MIXED::get(a));
         }
-        MIXED::add(tot, MIXED::mul(pre, MIXED::get(a)));
-    }
-    const cd v = MIXED::to_cd(MIXED::get(tot));
-    kacc ore, oim;
-    block_sum(v, ore, oim, red, buf);
-    if (threadIdx.x == 0) {
-        const double back = pow2d(max(min(t.A * e, 1000), -1000));
-        part[slice * t.n_chunks + chunk] = make_d4(ore.hi * back, ore.lo * back, oim.hi * back, oim.lo * back);
+        const cd v = MIXED::to_cd(MIXED::get(tot));
+        kacc ore, oim;
+        block_sum(v, ore, oim, red, buf);
+        if (threadIdx.x == 0) {
+            const double back = pow2d(max(min(t.A * e, 1000), -1000));
+            part[slice * t.n_chunks + chunk] = make_d4(ore.hi * back, ore.lo * back, oim.hi * back, oim.lo * back);
+        }
     }
 }
 
@@ -460,6 +510,7 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
 // time: the site's block entries are built in shared memory (diquark tables, then the
 // entries the plan uses), and the whole block factor tree is walked over them; the
 // site's compensated sum goes to its partial.  Complex double.
+template <bool REAL>
 __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, BlockTreeDev t,
                                                                 const double* __restrict__ U,
                                                                 const double* __restrict__ D, int64_t n_sites,
@@ -484,15 +535,7 @@ __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, Block
         cd grp = cd_make(0.0, 0.0);
         int in_grp = 0;
         for (int64_t u = threadIdx.x; u < t.n_units; u += blockDim.x) {
-            cd pre = cd_make(1.0, 0.0);
-            for (int k = 0; k < np; ++k) pre = cmul(pre, fs[__ldg(t.unit_pre + u * np + k)]);
-            cd s = cd_make(0.0, 0.0);
-            const int32_t l1 = __ldg(t.unit_leaf + u + 1);
-            for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
-                const double2 w = __ldg(t.leaf_wd + l);
-                cfma(s, cd_make(w.x, w.y), fs[__ldg(t.leaf_f + l)]);
-            }
-            cfma(grp, pre, s);
+            tree_unit<REAL>(t, u, np, fs, grp);
             if (++in_grp == 4) {
                 kacc_add(re, grp.re);
                 kacc_add(im, grp.im);
@@ -522,17 +565,19 @@ void project_shape(int n_f, int n_types, int64_t n_slices, int64_t V3, int sms, 
     const int per_cta = block_entries_per_cta(n_types);
     n_fc = (n_f + per_cta - 1) / per_cta;
     f_chunk = (n_f + n_fc - 1) / n_fc;
-    // at least four waves of one resident block per SM, tiles of at least 32 sites, and
-    // among up to four times that many tiles the count whose last wave is fullest
+    // one block per SM is resident: from four waves of tiles (or tiles of 32 sites) up to four times
+    // as many (or tiles of 16), the count with the least waves x (sites of a tile + 2), the 2
+    // for a tile's start and end.  Fewer, longer tiles would lose digits in the double-float
+    // running sums.  (4 slices of 4096 sites: 152 tiles a slice in four full waves, where 128
+    // left a third of the last wave empty.)
     const int64_t base = n_slices * n_fc;
-    const int64_t lo = (4LL * std::max(sms, 1) + base - 1) / base, cap = std::max<int64_t>(1, V3 / 32);
-    tiles = (int)std::max<int64_t>(1, std::min(lo, cap));
-    double best = 0.0;
-    for (int64_t t = std::min(lo, cap); t <= std::min(4 * lo, cap); ++t) {
-        const int64_t u = base * t;
-        const double eff = (double)u / (double)(((u + sms - 1) / sms) * sms);
-        if (eff > best + 1e-9) { best = eff; tiles = (int)t; }
-        if (eff >= 0.999) break;
+    const int64_t lo = std::max<int64_t>(1, std::min<int64_t>((4LL * std::max(sms, 1) + base - 1) / base, V3 / 32));
+    const int64_t cap = std::max<int64_t>(lo, std::min<int64_t>(4 * lo, V3 / 16));
+    int64_t best = INT64_MAX;
+    for (int64_t t = lo; t <= cap; ++t) {
+        const int64_t waves = (base * t + sms - 1) / std::max(sms, 1);
+        const int64_t cost = waves * ((V3 + t - 1) / t + 2);
+        if (cost < best) { best = cost; tiles = (int)t; }
     }
 }
 }  // namespace
@@ -577,29 +622,36 @@ cudaError_t launch_blocks_projected(const BlockDev& b, int prec, const double* U
     }
     ++*launches;
     const int64_t n = n_slices * b.n_f;
-    block_tile_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, n_slices, tiles, b.n_f, F);
+    block_tile_reduce_kernel<<<(unsigned)((n + 31) / 32), 32 * kReduceWarps, 0, s>>>(part, n_slices, tiles, b.n_f, F);
     ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_tree(const BlockTreeDev& t, int prec, const cd* F, int64_t n_slices, d4* part,
+cudaError_t launch_block_tree(const BlockTreeDev& t, int prec, const cd* F, int64_t n_slices, d4* part, int sms,
                               cudaStream_t s, int64_t* launches) {
     if (n_slices <= 0 || t.n_chunks <= 0) return cudaSuccess;
     const size_t smem = (size_t)t.n_f * 16;
-    const int64_t grid = (int64_t)t.n_chunks * n_slices;
-    if (prec == 1 && smem <= kSmemBudget) {
-        cudaError_t e = cudaFuncSetAttribute(block_tree_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        block_tree_df_kernel<<<(unsigned)grid, kTreeThreads, smem, s>>>(t, F, n_slices, part);
-    } else if (smem <= kSmemBudget) {
-        cudaError_t e = cudaFuncSetAttribute(block_tree_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        block_tree_kernel<true><<<(unsigned)grid, kTreeThreads, smem, s>>>(t, F, n_slices, part);
-    } else {
-        block_tree_kernel<false><<<(unsigned)grid, kTreeThreads, 0, s>>>(t, F, n_slices, part);
+    // blocks per slice: least waves x (chunks of a block + 1 for the slice's blocks)
+    int groups = 1;
+    int64_t best = INT64_MAX;
+    for (int g = 1; g <= t.n_chunks; ++g) {
+        const int64_t cost = ((n_slices * g + sms - 1) / std::max(sms, 1)) * ((t.n_chunks + g - 1) / g + 1);
+        if (cost < best) { best = cost; groups = g; }
     }
+    const int64_t grid = groups * n_slices;
+    auto launch = [&](auto kern, size_t bytes) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess) kern<<<(unsigned)grid, kTreeThreads, bytes, s>>>(t, F, n_slices, groups, part);
+        return e;
+    };
+    cudaError_t e;
+    if (prec == 1 && smem <= kSmemBudget)
+        e = t.real_w ? launch(block_tree_df_kernel<true>, smem) : launch(block_tree_df_kernel<false>, smem);
+    else if (smem <= kSmemBudget)
+        e = t.real_w ? launch(block_tree_kernel<true, true>, smem) : launch(block_tree_kernel<true, false>, smem);
+    else
+        e = t.real_w ? launch(block_tree_kernel<false, true>, 0) : launch(block_tree_kernel<false, false>, 0);
+    if (e != cudaSuccess) return e;
     ++*launches;
     return cudaGetLastError();
 }
@@ -613,11 +665,12 @@ cudaError_t launch_block_local(const BlockDev& b, const BlockTreeDev& t, const d
     if (n_sites <= 0) return cudaSuccess;
     const size_t smem = block_kernel_smem(b.n_f, b.n_types, true);
     if (smem > kSmemBudget) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(block_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = t.real_w ? block_local_kernel<true> : block_local_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int per_sm = std::max(1, (int)((227 * 1024) / (smem + 2 * 1024)));
     const int64_t grid = std::min<int64_t>(n_sites, (int64_t)sms * std::min(per_sm, 2048 / kThreads));
-    block_local_kernel<<<(unsigned)grid, kThreads, smem, s>>>(b, t, U, D, n_sites, part);
+    kern<<<(unsigned)grid, kThreads, smem, s>>>(b, t, U, D, n_sites, part);
     ++*launches;
     return cudaGetLastError();
 }

@@ -185,21 +185,34 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
             chunk_unit.push_back(u);
         }
         chunk_unit.push_back(n_units);
+        bool real_w = true;                       // (a weight exact in float has a zero low word as a double)
+        for (auto& x : h.w) real_w = real_w && x.imag() == 0.0;
         // one device allocation: entries | unit_pre | unit_leaf | leaf_f | leaf_w | chunk_unit
         size_t off = 0;
         auto place = [&](size_t bytes) { size_t o = off; off = (off + bytes + 255) / 256 * 256; return o; };
         const size_t o_e = place(entry.size() * 4), o_pre = place(h.unit_pre.size() * 2),
                      o_ul = place(h.unit_leaf.size() * 4), o_lf = place(h.leaf_f.size() * 2),
-                     o_lw = place(lw.size() * 8), o_lwd = place(h.w.size() * 16), o_cu = place(chunk_unit.size() * 8);
+                     o_lw = place(real_w ? 0 : lw.size() * 8), o_lwd = place(real_w ? 0 : h.w.size() * 16),
+                     o_rf = place(real_w ? h.w.size() * 8 : 0), o_rd = place(real_w ? h.w.size() * 8 : 0), o_cu = place(chunk_unit.size() * 8);
         std::vector<unsigned char> blob(std::max<size_t>(off, 256));
         std::memcpy(blob.data() + o_e, entry.data(), entry.size() * 4);
         if (!h.unit_pre.empty()) std::memcpy(blob.data() + o_pre, h.unit_pre.data(), h.unit_pre.size() * 2);
         std::memcpy(blob.data() + o_ul, h.unit_leaf.data(), h.unit_leaf.size() * 4);
         std::memcpy(blob.data() + o_lf, h.leaf_f.data(), h.leaf_f.size() * 2);
-        std::memcpy(blob.data() + o_lw, lw.data(), lw.size() * 8);
+        if (!real_w) std::memcpy(blob.data() + o_lw, lw.data(), lw.size() * 8);
         for (size_t i = 0; i < h.w.size(); ++i) {
             const double wd[2] = {h.w[i].real(), h.w[i].imag()};
-            std::memcpy(blob.data() + o_lwd + 16 * i, wd, 16);
+            if (!real_w) {
+                std::memcpy(blob.data() + o_lwd + 16 * i, wd, 16);
+                continue;
+            }
+            uint64_t bits;
+            std::memcpy(&bits, wd, 8);
+            uint32_t rf[2] = {h.leaf_f[i], 0u};
+            const uint32_t rd[2] = {h.leaf_f[i], (uint32_t)(bits >> 32)};
+            std::memcpy(rf + 1, &lw[i].x, 4);
+            std::memcpy(blob.data() + o_rf + 8 * i, rf, 8);
+            std::memcpy(blob.data() + o_rd + 8 * i, rd, 8);
         }
         std::memcpy(blob.data() + o_cu, chunk_unit.data(), chunk_unit.size() * 8);
         e = cudaMalloc(&P->dev, blob.size());
@@ -218,6 +231,9 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
         P->td.leaf_f = reinterpret_cast<const uint16_t*>(base + o_lf);
         P->td.leaf_w = reinterpret_cast<const float2*>(base + o_lw);
         P->td.leaf_wd = reinterpret_cast<const double2*>(base + o_lwd);
+        P->td.real_w = real_w ? 1 : 0;
+        P->td.leaf_rf = reinterpret_cast<const uint2*>(base + o_rf);
+        P->td.leaf_rd = reinterpret_cast<const uint2*>(base + o_rd);
         P->td.n_chunks = (int)n_chunks;
         P->td.chunk_unit = reinterpret_cast<const int64_t*>(base + o_cu);
     }
@@ -340,7 +356,7 @@ mbc_status mbc_block_correlator(mbc_block_plan* P, const void* U, const void* D,
     if (st != MBC_OK) return st;
     st = ensure(c, c->blk_tree, sizeof(d4) * (size_t)(n_slices * P->td.n_chunks), s);
     if (st != MBC_OK) return st;
-    e = launch_block_tree(P->td, P->hp.prec, (const cd*)c->blk_F.p, n_slices, (d4*)c->blk_tree.p, s, &c->launches);
+    e = launch_block_tree(P->td, P->hp.prec, (const cd*)c->blk_F.p, n_slices, (d4*)c->blk_tree.p, c->sms, s, &c->launches);
     if (e != cudaSuccess) return cuda_fail(c, e, "block tree launch");
     Geometry g{n_sets, T, (int64_t)P->td.n_chunks};
     Partials pt{(d4*)c->blk_tree.p, 1};
