@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(768, 1) egraph32_batch_kernel(const BatchItem3
 // err(t) > tol |C(t)|, the sites of the slice with the largest s_x are appended to the
 // recompute list -- those with s_x above the largest threshold tau for which the sites at
 // or below tau leave an estimate of at most tol |C(t)| / 2 (a recomputed site carries no
-// FP32 error; tau by bisection) -- skipping sites the site guard listed already (s_x = 0).
+// FP32 error) -- skipping sites the site guard listed already (s_x = 0).
 // C(t) here is the FP32 estimate with the momentum phase of the site sum.
 //
 // The threshold is found on the keys ceil(2^32 s_x / max s), three bits a pass, with the sums of
