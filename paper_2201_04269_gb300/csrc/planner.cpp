@@ -864,11 +864,16 @@ std::string validate_plan(const HostPlan& p) {
         if (d.blk_s0[i] < 0 || d.blk_s0[i] > d.blk_s1[i] || (size_t)d.blk_s1[i] > p.snk_w.size() || d.blk_r0[i] < 0 ||
             d.blk_r0[i] > d.blk_r1[i] || (size_t)d.blk_r1[i] > p.src_w.size())
             return "plan: direct block range out of range";
-    // factor tree: two levels, factor ids inside the minor tables, chunks inside the arrays
+    // factor tree: minors of n_u, n_d rows and columns out of 12, two levels, factor ids inside the
+    // minor tables, chunks inside the arrays
     const TreePlan& t = p.tree;
     if (t.children.size() != t.factors.size()) return "plan: tree arrays inconsistent";
     const int64_t n_um = (int64_t)t.minor_rows[0].size(), n_dm = (int64_t)t.minor_rows[1].size();
     if (t.minor_cols[0].size() != (size_t)n_um || t.minor_cols[1].size() != (size_t)n_dm) return "plan: tree minors inconsistent";
+    for (int f = 0; f < 2; ++f)
+        for (const std::vector<Mask>* v : {&t.minor_rows[f], &t.minor_cols[f]})
+            for (Mask m : *v)
+                if (m >> 12 || mask_size(m) != (f == 0 ? p.n_u : p.n_d)) return "plan: tree minor out of range";
     int64_t leaves = 0;
     for (size_t i = 1; i < t.factors.size(); ++i) {
         const int64_t f = t.factors[i];

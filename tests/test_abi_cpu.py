@@ -264,6 +264,69 @@ def test_damaged_plan_files_are_rejected_on_the_host(abi, hctx, tmp_path):
     assert detected > 0
 
 
+# the vectors of a plan file before the tree's minors, by element size; -1: a count of vectors of 24-byte
+# terms that follow (the canonical form per free index)
+PLAN_VECTORS = [1, 1, 16, 16, 8, 8, 16, 1, 1, 16, 2, 2, 2, 2, -1, -1, 24]
+
+
+def tree_minor_vectors(raw):
+    """Offset and count of the tree's four vectors of 16-bit index sets in a plan file's bytes: row
+    and column sets of the up minors, then of the down minors."""
+    def count(at):
+        return int.from_bytes(raw[at:at + 8], "little")
+    at = 8 + 5 * 4 + 16 + 1                      # magic, five ints, scale, the explicit flag
+    for size in PLAN_VECTORS:
+        n = count(at)
+        at += 8
+        if size > 0:
+            at += size * n
+            continue
+        for _ in range(n):
+            at += 8 + 24 * count(at)
+    out = []
+    for _ in range(4):
+        out.append((at + 8, count(at)))
+        at += 8 + 2 * out[-1][1]
+    return out
+
+
+def load_bytes(abi, ctx, path, raw):
+    """Load a plan file of these bytes; the error message when it is rejected, "" when it loads."""
+    open(path, "wb").write(bytes(raw))
+    try:
+        plan = abi.mbc_plan_load(ctx, path)
+    except abi.MbcError as e:
+        assert e.status in (1, 2, 3, 7)
+        return abi.mbc_last_error(ctx)
+    abi.mbc_plan_get_info(plan)
+    abi.mbc_plan_destroy(plan)
+    return ""
+
+
+@pytest.mark.parametrize("name", ["proton", "dinucleon_I"])
+@pytest.mark.parametrize("damage", [lambda m: m ^ 0xF000, lambda m: m | 0x8000, lambda m: m & (m - 1), lambda m: m | (m + 1),
+                                    lambda m: 0, lambda m: 0xFFF])
+def test_damaged_tree_minors_are_rejected(abi, hctx, tmp_path, name, damage):
+    """An index set of the tree's minors beyond 12 bits, or with more or fewer bits than its flavour
+    has quarks, is rejected on the host: the kernels' tables are built from the sets."""
+    plan, t = plan_of(abi, hctx, name, "tree", "mixed")
+    p = str(tmp_path / "t.mbcplan")
+    abi.mbc_plan_save(plan, p, hctx)
+    minors = {f: [abi.mbc_plan_get_minor(plan, f, m, n) for m in range(2)] for f, n in ((0, t["n_u"]), (1, t["n_d"]))}
+    abi.mbc_plan_destroy(plan)
+    raw = open(p, "rb").read()
+    assert load_bytes(abi, hctx, p, raw) == ""
+    for v, (at, n) in enumerate(tree_minor_vectors(raw)):
+        for m in (0, 1, n - 1):
+            buf = bytearray(raw)
+            here = at + 2 * m
+            mask = int.from_bytes(buf[here:here + 2], "little")
+            if m < 2:                            # (the offsets are those of the sets)
+                assert mask == sum(1 << int(i) for i in minors[v // 2][m][v % 2])
+            buf[here:here + 2] = damage(mask).to_bytes(2, "little")
+            assert "tree minor out of range" in load_bytes(abi, hctx, p, buf), (v, m)
+
+
 @pytest.mark.parametrize("name", ["dinucleon_I", "he3_I", "he3_II_s"])
 def test_minor_egraph_size_and_flops(abi, hctx, name):
     """The extracted Laplace plan costs less than one LU per minor, and the saturated
