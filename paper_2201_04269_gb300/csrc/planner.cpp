@@ -881,6 +881,8 @@ std::string validate_plan(const HostPlan& p) {
         if (t.children[i] == 0) ++leaves;
     }
     if (leaves != (int64_t)t.coefficients.size()) return "plan: tree leaves and coefficients differ";
+    for (size_t i = 1; i < t.factors.size(); i += 1 + (size_t)t.children[i])     // subtree by subtree
+        if ((size_t)t.children[i] >= t.factors.size() - i) return "plan: tree subtree out of range";
     if (t.chunk_leaf.size() != t.chunk_node.size() || t.chunk_count.size() != t.chunk_node.size())
         return "plan: tree chunks inconsistent";
     for (size_t c = 0; c < t.chunk_node.size(); ++c)

@@ -327,6 +327,24 @@ def test_damaged_tree_minors_are_rejected(abi, hctx, tmp_path, name, damage):
             assert "tree minor out of range" in load_bytes(abi, hctx, p, buf), (v, m)
 
 
+@pytest.mark.parametrize("more", [1, 2, 1 << 20, 0x7FFFFFFF])
+def test_damaged_tree_subtree_is_rejected(abi, hctx, tmp_path, more):
+    """A level-1 vertex of the tree with more children than the arrays hold is rejected."""
+    plan, _ = plan_of(abi, hctx, "proton", "tree", "mixed")
+    p = str(tmp_path / "t.mbcplan")
+    abi.mbc_plan_save(plan, p, hctx)
+    children = abi.mbc_plan_get_tree(plan)[1]
+    abi.mbc_plan_destroy(plan)
+    raw = bytearray(open(p, "rb").read())
+    at, n = tree_minor_vectors(raw)[3]
+    at += 2 * n                                  # the factors, then the child counts
+    at += 8 + 4 * int.from_bytes(raw[at:at + 8], "little") + 8
+    assert np.array_equal(np.frombuffer(raw, np.int32, len(children), at), children)
+    last = max(i for i in range(1, len(children)) if children[i] > 0)
+    raw[at + 4 * last:at + 4 * last + 4] = min(int(children[last]) + more, 0x7FFFFFFF).to_bytes(4, "little")
+    assert "tree subtree out of range" in load_bytes(abi, hctx, p, raw)
+
+
 @pytest.mark.parametrize("name", ["dinucleon_I", "he3_I", "he3_II_s"])
 def test_minor_egraph_size_and_flops(abi, hctx, name):
     """The extracted Laplace plan costs less than one LU per minor, and the saturated
