@@ -921,16 +921,27 @@ struct W {
     void raw(const void* p, size_t n) { if (ok && n && fwrite(p, 1, n, f) != n) ok = false; }
     template <class T> void pod(const T& v) { raw(&v, sizeof(T)); }
     template <class T> void vec(const std::vector<T>& v) { uint64_t n = v.size(); pod(n); raw(v.data(), n * sizeof(T)); }
+    template <class T> void vecs(const std::vector<T>& v) { uint64_t n = v.size(); pod(n); for (auto& x : v) vec(x); }
 };
 struct R {
     FILE* f;
+    uint64_t left;                              // bytes of the file not read yet: no vector is longer
     bool ok = true;
-    void raw(void* p, size_t n) { if (ok && n && fread(p, 1, n, f) != n) ok = false; }
+    void raw(void* p, size_t n) {
+        if (ok && n && (n > left || fread(p, 1, n, f) != n)) ok = false;
+        if (ok) left -= n;
+    }
     template <class T> void pod(T& v) { raw(&v, sizeof(T)); }
     template <class T> void vec(std::vector<T>& v) {
         uint64_t n = 0; pod(n);
-        if (!ok || n > (uint64_t)1 << 34) { ok = false; return; }
+        if (!ok || n > left / sizeof(T)) { ok = false; return; }
         v.resize(n); raw(v.data(), n * sizeof(T));
+    }
+    template <class T> void vecs(std::vector<T>& v) {
+        uint64_t n = 0; pod(n);
+        if (!ok || n > left / 8) { ok = false; return; }              // (each has at least its count)
+        v.resize(n);
+        for (auto& x : v) vec(x);
     }
 };
 template <class S> void minor_io(S& s, MinorPlan& m) {
@@ -943,8 +954,7 @@ template <class S> void plan_io(S& s, HostPlan& p) {
     s.vec(p.snk_idx); s.vec(p.src_idx); s.vec(p.snk_w); s.vec(p.src_w); s.vec(p.snk_off); s.vec(p.src_off); s.vec(p.proj);
     s.vec(p.ex_snk); s.vec(p.ex_src); s.vec(p.ex_w);
     for (int f = 0; f < 2; ++f) { s.vec(p.rows[f]); s.vec(p.cols[f]); }
-    uint64_t nj = p.snk_can.size(); s.pod(nj); p.snk_can.resize(nj); for (auto& v : p.snk_can) s.vec(v);
-    nj = p.src_can.size(); s.pod(nj); p.src_can.resize(nj); for (auto& v : p.src_can) s.vec(v);
+    s.vecs(p.snk_can); s.vecs(p.src_can);
     s.vec(p.terms);
     TreePlan& t = p.tree;
     for (int f = 0; f < 2; ++f) { s.vec(t.minor_rows[f]); s.vec(t.minor_cols[f]); }
@@ -974,7 +984,10 @@ std::string plan_write(const HostPlan& p, const std::string& path) {
 std::string plan_read(HostPlan& p, const std::string& path) {
     FILE* f = fopen(path.c_str(), "rb");
     if (!f) return "cannot open " + path;
-    R r{f};
+    // (a pipe has no size: no vector beyond 256 GB)
+    const long size = fseek(f, 0, SEEK_END) == 0 ? ftell(f) : -1;
+    if (size >= 0) rewind(f);
+    R r{f, size >= 0 ? (uint64_t)size : (uint64_t)1 << 38};
     char magic[8] = {0};
     r.raw(magic, 8);
     if (!r.ok || std::memcmp(magic, kMagic, 8) != 0) { fclose(f); return "not an mbc plan file (or another version): " + path; }

@@ -345,6 +345,27 @@ def test_damaged_tree_subtree_is_rejected(abi, hctx, tmp_path, more):
     assert "tree subtree out of range" in load_bytes(abi, hctx, p, raw)
 
 
+@pytest.mark.parametrize("byte", range(0, 8))
+def test_plan_file_counts_beyond_the_file_are_rejected(abi, hctx, tmp_path, byte):
+    """Any vector count of a plan file may be damaged in any byte: no allocation follows from a count
+    that the file cannot hold (the canonical form's lists of lists included)."""
+    plan, _ = plan_of(abi, hctx, "proton", "tree", "mixed")
+    p = str(tmp_path / "t.mbcplan")
+    abi.mbc_plan_save(plan, p, hctx)
+    abi.mbc_plan_destroy(plan)
+    raw = open(p, "rb").read()
+    at = 8 + 5 * 4 + 16 + 1
+    for size in PLAN_VECTORS:
+        buf = bytearray(raw)
+        buf[at + byte] ^= 0x55
+        assert load_bytes(abi, hctx, p, buf) != "", (at, byte)
+        n = int.from_bytes(raw[at:at + 8], "little")
+        at += 8
+        for _ in range(n if size < 0 else 0):
+            at += 8 + 24 * int.from_bytes(raw[at:at + 8], "little")
+        at += max(size, 0) * n
+
+
 @pytest.mark.parametrize("name", ["dinucleon_I", "he3_I", "he3_II_s"])
 def test_minor_egraph_size_and_flops(abi, hctx, name):
     """The extracted Laplace plan costs less than one LU per minor, and the saturated
