@@ -846,6 +846,7 @@ std::string validate_plan(const HostPlan& p) {
     for (int8_t v : p.ex_src) if (v < 0 || v > 11) return "plan: source index outside 0..11";
     if (p.ex_snk.size() != p.ex_w.size() * nq || p.ex_src.size() != p.ex_w.size() * nq) return "plan: explicit terms inconsistent";
     if (!p.explicit_terms) {
+        if (p.n_free < 0) return "plan: free index count out of range";
         if ((int)p.snk_off.size() != p.n_free + 1 || (int)p.src_off.size() != p.n_free + 1) return "plan: offsets size";
         for (int j = 0; j < p.n_free; ++j)
             if (p.snk_off[j] > p.snk_off[j + 1] || p.src_off[j] > p.src_off[j + 1]) return "plan: offsets decrease";
@@ -864,6 +865,9 @@ std::string validate_plan(const HostPlan& p) {
         if (d.blk_s0[i] < 0 || d.blk_s0[i] > d.blk_s1[i] || (size_t)d.blk_s1[i] > p.snk_w.size() || d.blk_r0[i] < 0 ||
             d.blk_r0[i] > d.blk_r1[i] || (size_t)d.blk_r1[i] > p.src_w.size())
             return "plan: direct block range out of range";
+    int64_t direct_terms = 0;
+    for (size_t i = 0; i < nb; ++i) direct_terms += (d.blk_s1[i] - d.blk_s0[i]) * (d.blk_r1[i] - d.blk_r0[i]);
+    if (d.index_size != (p.explicit_terms ? (int64_t)p.ex_w.size() : direct_terms)) return "plan: direct index count differs";
     // factor tree: minors of n_u, n_d rows and columns out of 12, two levels, factor ids inside the
     // minor tables, chunks inside the arrays
     const TreePlan& t = p.tree;

@@ -366,6 +366,21 @@ def test_plan_file_counts_beyond_the_file_are_rejected(abi, hctx, tmp_path, byte
         at += max(size, 0) * n
 
 
+@pytest.mark.parametrize("change", [1, -1, 1 << 40])
+def test_damaged_direct_index_count_is_rejected(abi, hctx, tmp_path, change):
+    """The direct sweep runs over as many terms as its blocks hold: another count is rejected."""
+    plan, _ = plan_of(abi, hctx, "proton", "direct", "fp64")
+    p = str(tmp_path / "t.mbcplan")
+    abi.mbc_plan_save(plan, p, hctx)
+    size = abi.mbc_plan_get_info(plan)["index_size"]
+    abi.mbc_plan_destroy(plan)
+    raw = bytearray(open(p, "rb").read())
+    at = len(raw) - 3 * 8 - 8                    # before the three flop counts
+    assert int.from_bytes(raw[at:at + 8], "little") == size
+    raw[at:at + 8] = (size + change).to_bytes(8, "little")
+    assert "direct index count differs" in load_bytes(abi, hctx, p, raw)
+
+
 @pytest.mark.parametrize("name", ["dinucleon_I", "he3_I", "he3_II_s"])
 def test_minor_egraph_size_and_flops(abi, hctx, name):
     """The extracted Laplace plan costs less than one LU per minor, and the saturated
