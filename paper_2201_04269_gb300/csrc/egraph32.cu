@@ -837,7 +837,10 @@ __global__ void __launch_bounds__(kGuardThreads) slice_guard_batch_kernel(const 
                      it.unit_begin, flag_count, flag_list, flag_cap, guard_keys);
 }
 
-// Threads and dynamic shared memory (keys) of the slice guard for slices of up to V3 sites.
+// Threads and dynamic shared memory (keys) of the slice guard for slices of up to V3 sites.  The kernels'
+// limit is always the largest size: it belongs to the kernel, not to a context, and a call of
+// small slices on another thread must not lower it before this one's launch.
+constexpr int kGuardSmemMax = kGuardKeys * (int)sizeof(unsigned int);
 inline int guard_threads(int64_t V3) { return (int)std::min<int64_t>(kGuardThreads, std::max<int64_t>(64, (V3 + 31) / 32 * 32)); }
 inline size_t guard_smem(int64_t V3) { return V3 <= kGuardKeys ? sizeof(unsigned int) * (size_t)V3 : 0; }
 
@@ -916,7 +919,7 @@ cudaError_t launch_egraph32(const Eg32Dev& d, const double* U, const double* D, 
     ++*launches;
     if (std::isinf(slice_tol) && slice_tol > 0) return cudaSuccess;      // slice guard off
     const size_t gs = guard_smem(g.V3);
-    e = cudaFuncSetAttribute(slice_guard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs);
+    e = cudaFuncSetAttribute(slice_guard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGuardSmemMax);
     if (e != cudaSuccess) return e;
     slice_guard_kernel<<<(unsigned)((int64_t)g.n_sets * g.T), guard_threads(g.V3), gs, s>>>(
         part, scale, g.V3, mom, slice_tol, flag_count, flag_list, (unsigned int)g.n_sites());
@@ -939,7 +942,7 @@ cudaError_t launch_egraph32_batch(const BatchItem32* items, int n_items, int64_t
     if (n_slices > 0) {
         // (slices larger than kGuardKeys recompute their keys and need no shared memory for them)
         const size_t gs = guard_smem(std::min<int64_t>(max_v3, kGuardKeys));
-        e = cudaFuncSetAttribute(slice_guard_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs);
+        e = cudaFuncSetAttribute(slice_guard_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGuardSmemMax);
         if (e != cudaSuccess) return e;
         slice_guard_batch_kernel<<<(unsigned)n_slices, guard_threads(max_v3), gs, s>>>(items, n_items, flag_count,
                                                                                       flag_list, (unsigned int)n_units);
