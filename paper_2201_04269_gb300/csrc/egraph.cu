@@ -332,9 +332,12 @@ __global__ void __launch_bounds__(384) egraph_kernel(EgraphDev d, const double* 
 }
 
 // Several (plan, fields) items in one persistent launch: work units are (item, site),
-// numbered item by item; a block takes units from the counter, finds the item by a
-// search over the unit offsets and evaluates the site with that item's plan.  Three
-// resident blocks of up to 384 threads per SM: the register cap this implies (56) costs a
+// numbered item by item; a block takes the unit of its own number, then units from the counter,
+// finds the item by a search over the unit offsets and evaluates the site with that item's
+// plan.  (Neighbouring blocks start on different SMs, so the units of a heavy item spread evenly; when
+// the first units came from the counter too, an SM of several small blocks could draw five of
+// them: dinucleon I and proton, 343 sites each in FP64, 2608 -> 1651 us.)  Three
+// resident blocks of 384 threads per SM: the register cap this implies (56) costs a
 // few spills of the per-item plan view, which the occupancy more than repays.
 template <class P>
 __global__ void __launch_bounds__(384, 3) egraph_batch_kernel(const BatchItem* __restrict__ items, int n_items,
@@ -350,8 +353,8 @@ __global__ void __launch_bounds__(384, 3) egraph_batch_kernel(const BatchItem* _
     typename P::V* K = kscratch + (size_t)blockIdx.x * kslot_values;
     // every unit, or (list mode) the units of a device list
     const int64_t n_work = list ? (int64_t)*list_n : n_units;
-    for (;;) {
-        if (threadIdx.x == 0) s_unit = atomicAdd(counter, 1u);
+    for (bool first = true;; first = false) {
+        if (threadIdx.x == 0) s_unit = first ? blockIdx.x : gridDim.x + atomicAdd(counter, 1u);
         __syncthreads();
         const int64_t work = s_unit;
         if (work >= n_work) break;

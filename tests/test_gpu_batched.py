@@ -273,3 +273,34 @@ def test_batched_workload_64_sets_full_size(ctx):
     print(f"batched 64 sets: {len(items)} items, {launches} launches, worst sampled-site error {worst:.2e}")
     for p in plans.values():
         p.destroy()
+
+
+@pytest.mark.parametrize("order", [("dinucleon_I", "proton"), ("proton", "dinucleon_I")])
+def test_small_batch_takes_no_longer_than_its_items(ctx, order):
+    """A batch of heavy and light FP64 sites, two to three heavy ones per SM, against the items one after
+    another: the heavy sites must spread over the SMs (the batch took 1.5 times as long when they
+    did not, and 0.95 times with them spread)."""
+    V3 = 343
+    U = torch.randn(1, 1, V3, 12, 12, dtype=torch.complex128, device="cuda")
+    D = torch.randn_like(U)
+    plans = [ctx.plan_operator(op, "egraph", "fp64") for op in order]
+    C = [torch.zeros(1, 1, dtype=torch.complex128, device="cuda") for _ in plans]
+    items = [dict(plan=p.handle, U=U, D=D, C=c, n_sets=1, T=1, V3=V3) for p, c in zip(plans, C)]
+
+    def ms(f):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        best = float("inf")
+        for k in range(8):                       # (the first three warm up)
+            a.record()
+            f()
+            b.record()
+            torch.cuda.synchronize()
+            if k >= 3:
+                best = min(best, a.elapsed_time(b))
+        return best
+
+    apart = ms(lambda: [p.correlator(U, D, c) for p, c in zip(plans, C)])
+    together = ms(lambda: ctx.batch(items))
+    for p in plans:
+        p.destroy()
+    assert together <= 1.25 * apart, (together, apart)
