@@ -664,6 +664,20 @@ def test_fp32_general_problems(ctx):
         plan.destroy()
 
 
+def test_fp64_builds_agree(ctx):
+    """FP64 e-graph calls of 3He I below and above the site count at which the build for more resident
+    blocks takes over (three blocks of 320 threads per SM): the same site values, bit for bit."""
+    plan = ctx.plan_operator("he3_I", "egraph", "fp64")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 3 * sms + 5
+    f = np.random.default_rng(14).standard_normal((2, 1, 1, n, 12, 12, 2)).view(np.complex128)[..., 0]
+    whole = run(plan, f[0], f[1])[1].ravel()
+    for a, b in ((0, 3 * sms), (3 * sms, n)):
+        part = run(plan, f[0][:, :, a:b], f[1][:, :, a:b])[1].ravel()
+        assert np.all(part != 0) and np.array_equal(part, whole[a:b])
+    plan.destroy()
+
+
 def test_fp32_empty_ragged_and_multiset(ctx):
     """MBC_PREC_FP32 on a ragged slice (37 sites), fewer sites than blocks (5), an empty lattice,
     and two sets in one call bit-identical to two separate calls."""
