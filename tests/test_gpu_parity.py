@@ -678,6 +678,37 @@ def test_fp64_builds_agree(ctx):
     plan.destroy()
 
 
+@pytest.mark.parametrize("n_u,n_d", [(2, 2), (2, 0), (0, 1), (1, 2), (2, 3)])
+@pytest.mark.parametrize("n_free,complex_w", [(1, False), (2, False), (3, False), (1, True)])
+def test_fp32_small_minors(ctx, n_u, n_d, n_free, complex_w):
+    """Both sides of the rule for two FP32 blocks per SM (minors up to 2 x 2, real weights, up to two free
+    indices), on more sites than one round of blocks, against the FP64 plan and, on some sites,
+    the oracle's index-set sum."""
+    from paper_2201_04269_gb300 import abi, Plan
+    rng = np.random.default_rng(1000 * n_u + 100 * n_d + 10 * n_free + complex_w)
+
+    def side():
+        idx = np.array([np.concatenate((rng.choice(12, n_u, replace=False), rng.choice(12, n_d, replace=False)))
+                        for _ in range(10 * n_free)]).astype(np.int8)
+        return idx, rng.standard_normal(10 * n_free) + (1j * rng.standard_normal(10 * n_free) if complex_w else 0j)
+    (si, sw), (ri, rw) = side(), side()
+    off = np.arange(n_free + 1) * 10
+    P = (rng.standard_normal((n_free, n_free)) + 0j)
+    plans = {p: Plan(ctx, abi.mbc_plan_create(ctx.handle, n_u, n_d, si, sw, off, ri, rw, off, P, 1.0, "egraph", p))
+             for p in ("fp32", "fp64")}
+    n_sites = 403
+    f = rng.standard_normal((2, 1, 1, n_sites, 12, 12, 2)).view(np.complex128)[..., 0]
+    S = {p: run(plan, f[0], f[1])[1].ravel() for p, plan in plans.items()}
+    assert np.max(np.abs(S["fp32"] - S["fp64"])) <= 1e-5 * np.max(np.abs(S["fp64"]))
+    snk = [(si[off[j]:off[j + 1]], sw[off[j]:off[j + 1]]) for j in range(n_free)]
+    src = [(ri[off[j]:off[j + 1]], rw[off[j]:off[j + 1]]) for j in range(n_free)]
+    n = n_u + n_d
+    ref = (-1) ** (n * (n - 1) // 2) * onat.direct(n_u, n_d, snk, src, P, f[0, 0, 0, :5], f[1, 0, 0, :5])
+    check(S["fp64"][:5], ref, "fp64")
+    for plan in plans.values():
+        plan.destroy()
+
+
 def test_fp32_empty_ragged_and_multiset(ctx):
     """MBC_PREC_FP32 on a ragged slice (37 sites), fewer sites than blocks (5), an empty lattice,
     and two sets in one call bit-identical to two separate calls."""

@@ -108,3 +108,36 @@ def test_slice_guard_sizes(ctx, V3):
     assert last == 2 * V3
     mixed.destroy()
     plan.destroy()
+
+
+def test_batched_slice_guard_of_mixed_slice_sizes(ctx):
+    """Items of one batch whose slices lie on both sides of the guard's block and key-table sizes are
+    guarded as in separate calls: the same C(t), bit for bit, and as many sites recomputed.  A
+    tolerance per size at which some slices are listed and some are not."""
+    from paper_2201_04269_gb300 import abi
+    items, plans, single, listed = [], [], [], 0
+    for V3, T in ((33, 40), (64, 40), (513, 20), (2048, 8), (40960, 3), (40961, 3)):
+        rng = np.random.default_rng(V3)
+        f = rng.standard_normal((2, 1, T, V3, 12, 12, 2)).view(np.complex128)[..., 0]
+        U, D = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in f)
+        plan = ctx.plan_operator("proton", "egraph", "fp32")
+        C = torch.zeros(1, T, dtype=torch.complex128, device="cuda")
+        n = 0
+        for tol in (2e-7, 3e-7, 5e-7, 8e-7, 1.2e-6):          # (the first at which not every slice is listed)
+            plan.set_guard(float("inf"), tol)
+            plan.correlator(U, D, C)
+            n = ctx.fp32_recomputed
+            if n < T * V3 // 4:
+                break
+        listed += n
+        single.append(C.cpu().numpy().copy())
+        items.append(dict(plan=plan.handle, U=U, D=D, n_sets=1, T=T, V3=V3, C=C))
+        plans.append(plan)
+    assert listed > 0
+    abi.mbc_batch(ctx.handle, items)
+    torch.cuda.synchronize()
+    assert ctx.fp32_recomputed == listed
+    for it, C in zip(items, single):
+        assert np.array_equal(it["C"].cpu().numpy(), C), it["V3"]
+    for plan in plans:
+        plan.destroy()

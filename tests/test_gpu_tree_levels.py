@@ -58,3 +58,28 @@ def test_tree_levels_match_direct(ctx, n_u, n_d, n_sets, n_terms, complex_w, pre
         # the sums of n_terms products cancel to about sqrt(n_terms) of them: compare to the
         # largest site value
         assert np.max(np.abs(got["tree"] - got["direct"])) <= tol * np.max(np.abs(got["direct"]))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_tree_of_more_sites_than_one_wave(ctx, prec):
+    """The tables of 3He I take 3.1 MB a site, so that 1500 sites run in three waves of at most 2 GB
+    with a shorter last one: the same site values, bit for bit, as in calls of one wave each."""
+    rng = np.random.default_rng(8)
+    plan = ctx.plan_operator("he3_I", "tree", prec)
+    wave = (2 << 30) // plan.info["scratch_bytes_per_site"] // 32 * 32
+    n = 1500
+    assert 2 * wave < n < 3 * wave
+    f = rng.standard_normal((2, 1, 1, n, 12, 12, 2)).view(np.complex128)[..., 0]
+    U, D = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in f)
+
+    def sites(a, b):
+        C = torch.zeros(1, 1, dtype=torch.complex128, device="cuda")
+        S = torch.zeros(1, 1, b - a, dtype=torch.complex128, device="cuda")
+        plan.correlator(U[:, :, a:b].contiguous(), D[:, :, a:b].contiguous(), C, S)
+        torch.cuda.synchronize()
+        return S.cpu().numpy().ravel()
+
+    whole = sites(0, n)
+    parts = np.concatenate([sites(a, min(a + 300, n)) for a in range(0, n, 300)])
+    plan.destroy()
+    assert np.all(whole != 0) and np.array_equal(whole, parts)
