@@ -60,7 +60,9 @@ __device__ __forceinline__ bool block_exponents(const double* __restrict__ a, co
     unsigned ma = 0u, mb = 0u;
     for (int i = threadIdx.x; i < 288; i += blockDim.x) {
         const double2 v = __ldg(reinterpret_cast<const double2*>(i < 144 ? a : b) + (i < 144 ? i : i - 144));
-        const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+        // (the lowest bit keeps a subnormal number below 2^-1042, whose high word is zero, from counting as zero)
+        const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu) |
+                           ((__double2loint(v.x) | __double2loint(v.y)) != 0);
         if (i < 144) ma = max(ma, m);
         else mb = max(mb, m);
     }

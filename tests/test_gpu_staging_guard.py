@@ -55,6 +55,30 @@ def test_staging_scales_exactly(ctx, algo, prec, shift):
     assert np.array_equal(np.ldexp(got[0].view(np.float64), k), got[1].view(np.float64))
 
 
+@pytest.mark.parametrize("tiny", [-1070, -1046, -1045, -1030])
+@pytest.mark.parametrize("algo,prec", [("egraph", "fp32"), ("egraph", "mixed"), ("tree", "mixed"), ("direct", "mixed")])
+def test_staging_of_subnormal_blocks(ctx, algo, prec, tiny):
+    """The same with a down block of subnormal numbers only: integers of up to three bits times
+    2^tiny, whose high words are all zero when the largest is below 2^-1042 (tiny up to -1045), and a site of
+    zeros, which stays zero."""
+    rng = np.random.default_rng(6)
+    f = rng.integers(-7, 8, (2, 1, 1, 33, 12, 12, 2)).astype(np.float64)
+    f[..., 0, 0, 0] = 7.0
+    f[1, 0, 0, 5] = 0.0
+    plan = ctx.plan_operator("proton", algo, prec)
+    if prec == "fp32":
+        plan.set_guard(float("inf"), float("inf"))
+    got = []
+    for a, b in ((0, 0), (500, tiny)):
+        z = np.stack((np.ldexp(f[0], a), np.ldexp(f[1], b))).view(np.complex128)[..., 0]
+        U, D = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in z)
+        got.append(sites(plan, U, D))
+    plan.destroy()
+    live = np.arange(33) != 5
+    assert np.all(got[0][live] != 0) and got[0][5] == 0
+    assert np.array_equal(np.ldexp(got[0].view(np.float64), 2 * 500 + tiny), got[1].view(np.float64))
+
+
 @pytest.mark.parametrize("algo,prec", [("egraph", "fp32"), ("egraph", "mixed")])
 @pytest.mark.parametrize("bad", [float("inf"), float("nan")])
 def test_staging_non_finite_site(ctx, algo, prec, bad):
