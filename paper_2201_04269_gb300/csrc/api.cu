@@ -218,7 +218,7 @@ std::string add_f32(const HostPlan& h, const F32Shape& shape, Eg32Dev& v, Blob& 
             shape.cluster < 0 || shape.cluster > 2)
             return "MBC_PREC_FP32 shape out of range (walkers 1..6, leaf batch 1..3 (1 with more than two free "
                    "indices), blocks per site 1..2)";
-        if (f32_smem(shape.walkers, shape.leaf_batch, pk_words, stack_vals, leaf_size) > 220 * 1024)
+        if (f32_smem(shape.walkers, shape.leaf_batch, pk_words, stack_vals, leaf_size) > kEgraph32SmemMax)
             return "MBC_PREC_FP32 shape needs more shared memory than a block has";
         W = shape.walkers;
         LB = shape.leaf_batch;
@@ -226,7 +226,7 @@ std::string add_f32(const HostPlan& h, const F32Shape& shape, Eg32Dev& v, Blob& 
     for (int w : {6, 4, 2, 1}) {
         if (W) break;
         for (int lb = max_lb; lb >= 1 && !W; --lb)
-            if (f32_smem(w, lb, pk_words, stack_vals, leaf_size) <= 220 * 1024) { W = w; LB = lb; }
+            if (f32_smem(w, lb, pk_words, stack_vals, leaf_size) <= kEgraph32SmemMax) { W = w; LB = lb; }
     }
     if (!W) return "MBC_PREC_FP32: the plan's tables do not fit shared memory";
     const int nrb = e.B.n ? (int)e.B.level_rows[e.B.n].size() : 1;
@@ -713,7 +713,7 @@ mbc_status upload(mbc_plan* P, const MinorLevels (&ml)[2]) {
     const int pk16 = (ed.A.size[ed.A.n] * ed.A.n + ed.B.size[ed.B.n] * ed.B.n + 3) / 4;
     auto resident = [](int values) { return std::min(225 * 1024 / (values * 16 + 3 * 1024), 2048 / 384); };
     // (they sit after the first 384 values, which the block sum reuses)
-    ed.stage_pk = base >= 384 && (base + pk16) * 16 <= 200 * 1024 &&
+    ed.stage_pk = base >= 384 && (base + pk16) * 16 <= kEgraphSmemMax &&
                   (h.prec == MBC_PREC_FP64 || resident(base + pk16) >= resident(base));
     ed.smem_values = std::max(base + (ed.stage_pk ? pk16 : 0), 384);      // (the block sum takes a value per thread)
     return upload_f32(P);
@@ -789,7 +789,7 @@ mbc_status finish_plan(mbc_ctx* ctx, mbc_plan* P, mbc_plan** out) {
         delete P;
         return st;
     }
-    if (h.algo == MBC_ALGO_EGRAPH && P->ed.smem_values * 16 > 200 * 1024) {
+    if (h.algo == MBC_ALGO_EGRAPH && P->ed.smem_values * 16 > kEgraphSmemMax) {
         cudaFree(P->dev);
         if (P->dev32) cudaFree(P->dev32);
         delete P;

@@ -27,7 +27,7 @@ constexpr int kQ = 144;           // one 12 x 12 propagator
 constexpr int kDq = 432;          // one diquark table [c][s][s2]
 constexpr int kThreads = 512;
 constexpr int kTreeThreads = 512;
-constexpr size_t kSmemBudget = 200 * 1024;
+constexpr int kSmemBudget = 200 * 1024;       // also the kernels' limit, whatever a call needs (as in device.cuh)
 
 __device__ __forceinline__ cd cmul(cd a, cd b) { return cd_make(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
 __device__ __forceinline__ void cfma(cd& acc, cd a, cd b) {
@@ -609,13 +609,12 @@ cudaError_t launch_blocks_projected(const BlockDev& b, int prec, const double* U
     const int64_t units = n_slices * tiles * n_fc;
     const int px = p ? p[0] : 0, py = p ? p[1] : 0, pz = p ? p[2] : 0;
     if (prec == 0) {
-        cudaError_t e = cudaFuncSetAttribute(block_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(block_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e != cudaSuccess) return e;
         block_project_kernel<<<(unsigned)units, kThreads, smem, s>>>(b, U, D, V3, L, px, py, pz, tiles, f_chunk, n_fc,
                                                                      part);
     } else {
-        cudaError_t e = cudaFuncSetAttribute(block_project_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(block_project_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e != cudaSuccess) return e;
         block_project_df_kernel<<<(unsigned)units, kThreads, smem, s>>>(b, U, D, V3, L, px, py, pz, tiles, f_chunk,
                                                                         n_fc, part);
@@ -640,7 +639,7 @@ cudaError_t launch_block_tree(const BlockTreeDev& t, int prec, const cd* F, int6
     }
     const int64_t grid = groups * n_slices;
     auto launch = [&](auto kern, size_t bytes) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e == cudaSuccess) kern<<<(unsigned)grid, kTreeThreads, bytes, s>>>(t, F, n_slices, groups, part);
         return e;
     };
@@ -666,7 +665,7 @@ cudaError_t launch_block_local(const BlockDev& b, const BlockTreeDev& t, const d
     const size_t smem = block_kernel_smem(b.n_f, b.n_types, true);
     if (smem > kSmemBudget) return cudaErrorInvalidValue;
     auto kern = t.real_w ? block_local_kernel<true> : block_local_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     if (e != cudaSuccess) return e;
     const int per_sm = std::max(1, (int)((227 * 1024) / (smem + 2 * 1024)));
     const int64_t grid = std::min<int64_t>(n_sites, (int64_t)sms * std::min(per_sm, 2048 / kThreads));

@@ -76,6 +76,12 @@ struct TreeDev {
 };
 static constexpr int kTreeSplit = 8;
 
+// Largest dynamic shared memory of a block (plans beyond it are refused).  A kernel's limit belongs to the
+// kernel, which all contexts of the process share, so every launch sets it to the same largest
+// size: with each call's own size, another thread's smaller call could lower it between this
+// one's setting and its launch, which then failed.
+static constexpr int kEgraphSmemMax = 200 * 1024, kEgraph32SmemMax = 220 * 1024;
+
 // ---------------------------------------------------------------- e-graph plan
 struct MinorDev {
     int n;

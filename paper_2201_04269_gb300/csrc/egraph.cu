@@ -383,8 +383,8 @@ cudaError_t launch_egraph_batch(const BatchItem* items, int n_items, int64_t n_u
                                 int64_t* launches) {
     if (n_units == 0) return cudaSuccess;
     cudaError_t e;
-    if (prec == 0) e = cudaFuncSetAttribute(egraph_batch_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    else e = cudaFuncSetAttribute(egraph_batch_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (prec == 0) e = cudaFuncSetAttribute(egraph_batch_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
+    else e = cudaFuncSetAttribute(egraph_batch_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     if (e != cudaSuccess) return e;
     grid = (int)std::min<int64_t>(n_units, grid);
     e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
@@ -404,8 +404,7 @@ cudaError_t launch_egraph_batch_list(const BatchItem* items, int n_items, int64_
                                      const unsigned int* list, const unsigned int* list_n, cudaStream_t s,
                                      int64_t* launches) {
     if (n_items == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(egraph_batch_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(egraph_batch_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
@@ -427,8 +426,8 @@ cudaError_t launch_egraph(const EgraphDev& d, int prec, const double* U, const d
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     auto fp64 = grid > sms * (65536 / (56 * threads)) ? egraph_kernel<FP64, 4> : egraph_kernel<FP64>;
-    if (prec == 0) e = cudaFuncSetAttribute(fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    else e = cudaFuncSetAttribute(egraph_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (prec == 0) e = cudaFuncSetAttribute(fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
+    else e = cudaFuncSetAttribute(egraph_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
@@ -444,7 +443,7 @@ cudaError_t launch_egraph_list(const EgraphDev& d, const double* U, const double
                                int grid, unsigned int* counter, void* kscratch, const unsigned int* list,
                                const unsigned int* list_n, int64_t n_sites, cudaStream_t s, int64_t* launches) {
     const size_t smem = egraph_smem_bytes(d, 1);
-    cudaError_t e = cudaFuncSetAttribute(egraph_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(egraph_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;

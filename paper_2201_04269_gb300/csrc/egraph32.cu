@@ -837,9 +837,8 @@ __global__ void __launch_bounds__(kGuardThreads) slice_guard_batch_kernel(const 
                      it.unit_begin, flag_count, flag_list, flag_cap, guard_keys);
 }
 
-// Threads and dynamic shared memory (keys) of the slice guard for slices of up to V3 sites.  The kernels'
-// limit is always the largest size: it belongs to the kernel, not to a context, and a call of
-// small slices on another thread must not lower it before this one's launch.
+// Threads and dynamic shared memory (keys) of the slice guard for slices of up to V3 sites; the kernels'
+// limit is always the largest size (as in device.cuh).
 constexpr int kGuardSmemMax = kGuardKeys * (int)sizeof(unsigned int);
 inline int guard_threads(int64_t V3) { return (int)std::min<int64_t>(kGuardThreads, std::max<int64_t>(64, (V3 + 31) / 32 * 32)); }
 inline size_t guard_smem(int64_t V3) { return V3 <= kGuardKeys ? sizeof(unsigned int) * (size_t)V3 : 0; }
@@ -849,7 +848,7 @@ inline size_t guard_smem(int64_t V3) { return V3 <= kGuardKeys ? sizeof(unsigned
 template <class K, class... Args>
 cudaError_t launch_clusters(K kern, int cs, int walkers, int smem, int64_t want, int max_grid, cudaStream_t s,
                             Args... args) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraph32SmemMax);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(walkers * kWalker);

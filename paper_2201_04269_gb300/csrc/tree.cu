@@ -250,12 +250,9 @@ cudaError_t launch_tree(const TreeDev& d, int prec, const double* U, const doubl
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = (size_t)kTreeSites * kPad * 16;
-    static bool attr_set[2] = {false, false};
-    if (!attr_set[prec]) {
-        if (prec == 0) cudaFuncSetAttribute(minor_table_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        else cudaFuncSetAttribute(minor_table_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr_set[prec] = true;
-    }
+    cudaError_t attr = prec == 0 ? cudaFuncSetAttribute(minor_table_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                 : cudaFuncSetAttribute(minor_table_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr != cudaSuccess) return attr;
     cudaMemsetAsync(exps, 0, sizeof(int) * 2 * (size_t)std::min(total, scratch_sites), s);
     for (int64_t site0 = 0; site0 < total; site0 += scratch_sites) {
         const int64_t n = std::min(scratch_sites, total - site0);

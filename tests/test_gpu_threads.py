@@ -34,12 +34,17 @@ class Caller:
         self.U, self.D = fields(T, L ** 3)
         self.C = torch.zeros(1, T, dtype=torch.complex128, device="cuda")
         s = self.stream.cuda_stream
-        self.plan = self.ctx.plan_operator(op, "egraph", prec)
-        if kind == "batch":
-            items = [dict(plan=self.plan.handle, U=self.U, D=self.D, n_sets=1, T=T, V3=L ** 3, C=self.C)]
-            self.call = lambda: self.ctx.batch(items, s)
+        if kind in ("blocks", "blocks_local"):
+            self.plan = self.ctx.block_plan(op, prec)
+            self.call = (lambda: self.plan.correlator(self.U, self.D, self.C, L, stream=s)) if kind == "blocks" else \
+                (lambda: self.plan.correlator_local(self.U, self.D, self.C, stream=s))
         else:
-            self.call = lambda: self.plan.correlator(self.U, self.D, self.C, stream=s)
+            self.plan = self.ctx.plan_operator(op, "egraph", prec)
+            if kind == "batch":
+                items = [dict(plan=self.plan.handle, U=self.U, D=self.D, n_sets=1, T=T, V3=L ** 3, C=self.C)]
+                self.call = lambda: self.ctx.batch(items, s)
+            else:
+                self.call = lambda: self.plan.correlator(self.U, self.D, self.C, stream=s)
         torch.cuda.synchronize()
         self.call()
         torch.cuda.synchronize()
@@ -64,9 +69,18 @@ GUARDS = [
     ("call", ("proton", "fp32", 1, 24), ("proton", "fp32", 1, 4)),             # slice guard: 55 KB and 256 bytes
     ("batch", ("proton", "fp32", 1, 24), ("proton", "fp32", 1, 4)),            # its batched form
 ]
+PLANS = [
+    ("call", ("he3_II_s", "fp32", 1, 1), ("he3_I", "fp32", 1, 1)),             # FP32 kernel
+    ("call", ("dinucleon_I", "mixed", 1, 2), ("proton", "mixed", 1, 2)),       # double-float and FP64 kernels
+    ("call", ("dinucleon_I", "fp64", 1, 2), ("proton", "fp64", 1, 2)),
+    ("batch", ("dinucleon_I", "mixed", 1, 2), ("proton", "mixed", 1, 2)),
+    ("blocks", ("dinucleon_I", "fp64", 1, 2), ("proton", "fp64", 1, 2)),       # projection and block tree
+    ("blocks", ("dinucleon_I", "mixed", 1, 2), ("proton", "mixed", 1, 2)),
+    ("blocks_local", ("dinucleon_I", "fp64", 1, 2), ("proton", "fp64", 1, 2)),
+]
 
 
-@pytest.mark.parametrize("kind,a,b", GUARDS)
+@pytest.mark.parametrize("kind,a,b", GUARDS + PLANS)
 def test_threads_do_not_share_shared_memory_limits(kind, a, b):
     """A kernel's shared-memory limit belongs to the kernel, not to a context: no call may be refused
     because another thread's call of a smaller size came in between."""
