@@ -32,7 +32,7 @@ struct BlockTreeDev {
     int64_t n_units;
     const uint16_t* unit_pre;      // [n_units][A - 1]
     const int32_t* unit_leaf;      // [n_units + 1]
-    // leaves: compact factor and integer-valued weight (exact in float).  Real weights (every operator
+    // leaves: compact factor and integer-valued weight (leaf_weight).  Real weights (every operator
     // of the library): (factor, float bits) for the double-float tree, (factor, high word of the
     // double, whose low word is zero) for FP64; complex ones: factor, weight
     int real_w;

@@ -65,4 +65,9 @@ struct BlockHostPlan {
 };
 std::string plan_blocks(BlockHostPlan& bp);                // blocks_planner.cpp
 
+// A leaf weight as the device trees hold it: float bits (double-float tree) and the high word of the
+// double (FP64 tree).  False unless the weight is real, exact in a float and of at most 21
+// significant bits (a double's high word holds 20 fraction bits, a float 23).
+bool leaf_weight(cplx w, uint32_t& float_bits, uint32_t& high_word);   // blocks_planner.cpp
+
 }  // namespace mbc

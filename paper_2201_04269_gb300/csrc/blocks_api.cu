@@ -157,9 +157,10 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
     std::vector<float2> lw(h.w.size());
     for (size_t i = 0; i < h.w.size(); ++i) {
         lw[i] = make_float2((float)h.w[i].real(), (float)h.w[i].imag());
-        if ((double)lw[i].x != h.w[i].real() || (double)lw[i].y != h.w[i].imag()) {
+        uint32_t float_bits, high_word;
+        if (!leaf_weight(h.w[i], float_bits, high_word)) {
             delete P;
-            return fail(c, MBC_UNSUPPORTED, "merged block weight not exact in float");
+            return fail(c, MBC_UNSUPPORTED, "merged block weight not a real number of at most 21 bits");
         }
     }
     if (c->device >= 0 && !h.w.empty()) {
@@ -185,7 +186,7 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
             chunk_unit.push_back(u);
         }
         chunk_unit.push_back(n_units);
-        bool real_w = true;                       // (a weight exact in float has a zero low word as a double)
+        bool real_w = true;
         for (auto& x : h.w) real_w = real_w && x.imag() == 0.0;
         // one device allocation: entries | unit_pre | unit_leaf | leaf_f | leaf_w | chunk_unit
         size_t off = 0;

@@ -277,4 +277,14 @@ std::string plan_blocks(BlockHostPlan& bp) {
     return "";
 }
 
+bool leaf_weight(cplx w, uint32_t& float_bits, uint32_t& high_word) {
+    const double x = w.real();
+    const float f = (float)x;
+    uint64_t bits;
+    std::memcpy(&bits, &x, 8);
+    std::memcpy(&float_bits, &f, 4);
+    high_word = (uint32_t)(bits >> 32);
+    return w.imag() == 0.0 && (double)f == x && (uint32_t)bits == 0u;
+}
+
 }  // namespace mbc

@@ -2,10 +2,17 @@
 merged block form of each library operator agrees with the oracle's construction
 (arXiv 2201.04269 Sec. 3), term by term, and the argument checks of the block entry
 points reject bad input without touching a device."""
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 
 from oracle import blocks as obl
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2201_04269_gb300", "csrc")
 
 
 @pytest.fixture(scope="module")
@@ -98,3 +105,18 @@ def test_shared_leaf_sums_match_oracle(abi, hctx, name):
     assert info["shared_sums"] == len(sums)
     assert info["shared_sum_terms"] == sum(len(s) for s in sums)
     abi.mbc_block_plan_destroy(plan)
+
+
+def test_leaf_weights_are_exact(tmp_path):
+    """tests/block_weights_check.cpp: the device trees' leaf records hold every accepted weight
+    exactly, larger odd integers, fractions and complex weights are refused, and the operators'
+    weights are accepted."""
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no g++")
+    exe = str(tmp_path / "block_weights_check")
+    subprocess.run([cxx, "-O2", "-std=c++17", f"-I{CSRC}", os.path.join(ROOT, "tests", "block_weights_check.cpp"),
+                    os.path.join(CSRC, "blocks_planner.cpp"), os.path.join(CSRC, "planner.cpp"), "-o", exe],
+                   check=True, capture_output=True, timeout=600)
+    out = subprocess.run([exe] + [str(op) for op in range(7)], capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0 and out.stdout.startswith("OK"), out.stdout + out.stderr
