@@ -375,26 +375,20 @@ __global__ void __launch_bounds__(32 * kReduceWarps) block_tile_reduce_kernel(co
 }
 
 // One unit of the block factor tree in complex double: the product of its path's factors times
-// the weighted sum of its leaves, added to grp.  Real weights (all of the library's) take
-// half the multiply-adds and one 8-byte record a leaf: dinucleon I at the local sink, 4096 sites,
-// 3.12 -> 2.36 ms, bound by the FP64 pipe.
-template <bool REAL>
+// the weighted sum of its leaves, added to grp.  The weights are real, which takes half the
+// multiply-adds of complex ones and one 8-byte record a leaf: dinucleon I at the local sink, 4096
+// sites, 3.12 -> 2.36 ms, bound by the FP64 pipe.
 __device__ __forceinline__ void tree_unit(const BlockTreeDev& t, int64_t u, int np, const cd* Fs, cd& grp) {
     cd pre = np ? Fs[__ldg(t.unit_pre + u * np)] : cd_make(1.0, 0.0);
     for (int k = 1; k < np; ++k) pre = cmul(pre, Fs[__ldg(t.unit_pre + u * np + k)]);
     cd s = cd_make(0.0, 0.0);
     const int32_t l1 = __ldg(t.unit_leaf + u + 1);
     for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
-        if (REAL) {
-            const uint2 r = __ldg(t.leaf_rd + l);
-            const double w = __hiloint2double((int)r.y, 0);
-            const cd f = Fs[r.x];
-            s.re = fma(w, f.re, s.re);
-            s.im = fma(w, f.im, s.im);
-        } else {
-            const double2 w = __ldg(t.leaf_wd + l);
-            cfma(s, cd_make(w.x, w.y), Fs[__ldg(t.leaf_f + l)]);
-        }
+        const uint2 r = __ldg(t.leaf_rd + l);
+        const double w = __hiloint2double((int)r.y, 0);
+        const cd f = Fs[r.x];
+        s.re = fma(w, f.re, s.re);
+        s.im = fma(w, f.im, s.im);
     }
     cfma(grp, pre, s);
 }
@@ -404,7 +398,6 @@ __device__ __forceinline__ void tree_unit(const BlockTreeDev& t, int64_t u, int 
 // projected blocks are loaded (double-float: scaled and split, FP64 arithmetic worth a chunk's
 // walk) once for all of them (launch_block_tree chooses the groups).  3He_II-s double-float, 4 slices: 680 ->
 // 503 us against one block per chunk.
-template <bool SMEM, bool REAL>
 __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t, const cd* __restrict__ F,
                                                                    int64_t n_slices, int groups,
                                                                    d4* __restrict__ part) {
@@ -412,13 +405,9 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
     __shared__ double red[4];
     __shared__ cd buf[kTreeThreads];
     const int64_t slice = blockIdx.x % n_slices;
-    const cd* Fs = F + slice * t.n_f;
-    if (SMEM) {
-        cd* fs = reinterpret_cast<cd*>(smem_raw);
-        for (int i = threadIdx.x; i < t.n_f; i += blockDim.x) fs[i] = Fs[i];
-        __syncthreads();
-        Fs = fs;
-    }
+    cd* fs = reinterpret_cast<cd*>(smem_raw);
+    for (int i = threadIdx.x; i < t.n_f; i += blockDim.x) fs[i] = F[slice * t.n_f + i];
+    __syncthreads();
     const int np = t.A - 1;
     for (int chunk = (int)(blockIdx.x / n_slices); chunk < t.n_chunks; chunk += groups) {
         kacc re = {0.0, 0.0}, im = {0.0, 0.0};
@@ -426,7 +415,7 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
         cd grp = cd_make(0.0, 0.0);
         int in_grp = 0;
         for (int64_t u = t.chunk_unit[chunk] + threadIdx.x; u < t.chunk_unit[chunk + 1]; u += blockDim.x) {
-            tree_unit<REAL>(t, u, np, Fs, grp);
+            tree_unit(t, u, np, fs, grp);
             if (++in_grp == 4) {
                 kacc_add(re, grp.re);
                 kacc_add(im, grp.im);
@@ -446,7 +435,6 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_kernel(BlockTreeDev t
 // exact power of two 2^-e (e from the largest |re|, |im| among them) into (hi, lo) float
 // pairs in shared memory; a term of A factors then carries 2^(A e), restored in double
 // on the block's partial sum.
-template <bool REAL>
 __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDev t, const cd* __restrict__ F,
                                                                       int64_t n_slices, int groups,
                                                                       d4* __restrict__ part) {
@@ -481,18 +469,11 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
             MIXED::acc_zero(a);
             const int32_t l1 = __ldg(t.unit_leaf + u + 1);
             for (int32_t l = __ldg(t.unit_leaf + u); l < l1; ++l) {
-                if (REAL) {
-                    const uint2 r = __ldg(t.leaf_rf + l);
-                    dacc2_fma_f(a.x, __uint_as_float(r.y), fs[r.x]);
-                    continue;
-                }
-                const float2 w = __ldg(t.leaf_w + l);
-                const cdf f = fs[__ldg(t.leaf_f + l)];
-                // (w.x + i w.y) f with float weights (exact products by error-free transformation)
-                dacc2_fma_f(a.x, w.x, f);
-                dacc2_fma_f(a.y, w.y, f);
+                const uint2 r = __ldg(t.leaf_rf + l);
+                // (exact product of a float weight by error-free transformation)
+                dacc2_fma_f(a.x, __uint_as_float(r.y), fs[r.x]);
             }
-            MIXED::fma(tot, pre, REAL ? MIXED::get_s(a) : MIXED::get(a));
+            MIXED::fma(tot, pre, MIXED::get_s(a));
         }
         const cd v = MIXED::to_cd(MIXED::get(tot));
         kacc ore, oim;
@@ -510,7 +491,6 @@ __global__ void __launch_bounds__(kTreeThreads) block_tree_df_kernel(BlockTreeDe
 // time: the site's block entries are built in shared memory (diquark tables, then the
 // entries the plan uses), and the whole block factor tree is walked over them; the
 // site's compensated sum goes to its partial.  Complex double.
-template <bool REAL>
 __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, BlockTreeDev t,
                                                                 const double* __restrict__ U,
                                                                 const double* __restrict__ D, int64_t n_sites,
@@ -535,7 +515,7 @@ __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, Block
         cd grp = cd_make(0.0, 0.0);
         int in_grp = 0;
         for (int64_t u = threadIdx.x; u < t.n_units; u += blockDim.x) {
-            tree_unit<REAL>(t, u, np, fs, grp);
+            tree_unit(t, u, np, fs, grp);
             if (++in_grp == 4) {
                 kacc_add(re, grp.re);
                 kacc_add(im, grp.im);
@@ -553,6 +533,8 @@ __global__ void __launch_bounds__(kThreads) block_local_kernel(BlockDev b, Block
 }
 
 }  // namespace
+
+bool block_tree_fits(int n_f) { return (size_t)n_f * 16 <= (size_t)kSmemBudget; }
 
 int block_entries_per_cta(int n_types) { return (int)(kSmemBudget / 16) - 2 * kQ - n_types * kDq; }
 
@@ -638,18 +620,12 @@ cudaError_t launch_block_tree(const BlockTreeDev& t, int prec, const cd* F, int6
         if (cost < best) { best = cost; groups = g; }
     }
     const int64_t grid = groups * n_slices;
-    auto launch = [&](auto kern, size_t bytes) {
+    auto launch = [&](auto kern) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        if (e == cudaSuccess) kern<<<(unsigned)grid, kTreeThreads, bytes, s>>>(t, F, n_slices, groups, part);
+        if (e == cudaSuccess) kern<<<(unsigned)grid, kTreeThreads, smem, s>>>(t, F, n_slices, groups, part);
         return e;
     };
-    cudaError_t e;
-    if (prec == 1 && smem <= kSmemBudget)
-        e = t.real_w ? launch(block_tree_df_kernel<true>, smem) : launch(block_tree_df_kernel<false>, smem);
-    else if (smem <= kSmemBudget)
-        e = t.real_w ? launch(block_tree_kernel<true, true>, smem) : launch(block_tree_kernel<true, false>, smem);
-    else
-        e = t.real_w ? launch(block_tree_kernel<false, true>, 0) : launch(block_tree_kernel<false, false>, 0);
+    const cudaError_t e = prec == 1 ? launch(block_tree_df_kernel) : launch(block_tree_kernel);
     if (e != cudaSuccess) return e;
     ++*launches;
     return cudaGetLastError();
@@ -664,12 +640,11 @@ cudaError_t launch_block_local(const BlockDev& b, const BlockTreeDev& t, const d
     if (n_sites <= 0) return cudaSuccess;
     const size_t smem = block_kernel_smem(b.n_f, b.n_types, true);
     if (smem > kSmemBudget) return cudaErrorInvalidValue;
-    auto kern = t.real_w ? block_local_kernel<true> : block_local_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    cudaError_t e = cudaFuncSetAttribute(block_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     if (e != cudaSuccess) return e;
     const int per_sm = std::max(1, (int)((227 * 1024) / (smem + 2 * 1024)));
     const int64_t grid = std::min<int64_t>(n_sites, (int64_t)sms * std::min(per_sm, 2048 / kThreads));
-    kern<<<(unsigned)grid, kThreads, smem, s>>>(b, t, U, D, n_sites, part);
+    block_local_kernel<<<(unsigned)grid, kThreads, smem, s>>>(b, t, U, D, n_sites, part);
     ++*launches;
     return cudaGetLastError();
 }

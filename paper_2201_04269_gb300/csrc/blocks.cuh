@@ -32,15 +32,10 @@ struct BlockTreeDev {
     int64_t n_units;
     const uint16_t* unit_pre;      // [n_units][A - 1]
     const int32_t* unit_leaf;      // [n_units + 1]
-    // leaves: compact factor and integer-valued weight (leaf_weight).  Real weights (every operator
-    // of the library): (factor, float bits) for the double-float tree, (factor, high word of the
-    // double, whose low word is zero) for FP64; complex ones: factor, weight
-    int real_w;
+    // leaves: compact factor and real weight (leaf_weight): float bits for the double-float tree, the high
+    // word of the double, whose low word is zero, for FP64
     const uint2* leaf_rf;
     const uint2* leaf_rd;
-    const uint16_t* leaf_f;        // [leaves]
-    const float2* leaf_w;          // [leaves]
-    const double2* leaf_wd;        // [leaves] the same in double: FP64 tree
     int n_chunks;
     const int64_t* chunk_unit;     // [n_chunks + 1]
 };
@@ -65,6 +60,8 @@ cudaError_t launch_blocks_projected(const BlockDev& b, int prec, const double* U
 // plan's block entries do not fit shared memory.
 cudaError_t launch_block_local(const BlockDev& b, const BlockTreeDev& t, const double* U, const double* D,
                                int64_t n_sites, d4* part, int sms, cudaStream_t s, int64_t* launches);
+// Whether a slice's projected blocks fit a block's shared memory for the tree.
+bool block_tree_fits(int n_f);
 // Factor tree over projected blocks: part [n_slices][t.n_chunks] compensated partial sums;
 // prec 0 in complex double, 1 in double-float (the slice's blocks scaled by a power of two).
 cudaError_t launch_block_tree(const BlockTreeDev& t, int prec, const cd* F, int64_t n_slices, d4* part, int sms,

@@ -2,6 +2,7 @@
 // momentum-projected blocks (arXiv 2201.04269 Sec. 2), block plans and the block form of
 // the correlator (Secs. 3-4).
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -154,14 +155,15 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
     }
     if (!err.empty()) { delete P; return fail(c, MBC_INVALID_ARG, err); }
     BlockHostPlan& h = P->hp;
-    std::vector<float2> lw(h.w.size());
-    for (size_t i = 0; i < h.w.size(); ++i) {
-        lw[i] = make_float2((float)h.w[i].real(), (float)h.w[i].imag());
-        uint32_t float_bits, high_word;
-        if (!leaf_weight(h.w[i], float_bits, high_word)) {
+    std::vector<std::array<uint32_t, 2>> lw(h.w.size());      // float bits, high word of the double
+    for (size_t i = 0; i < h.w.size(); ++i)
+        if (!leaf_weight(h.w[i], lw[i][0], lw[i][1])) {
             delete P;
             return fail(c, MBC_UNSUPPORTED, "merged block weight not a real number of at most 21 bits");
         }
+    if (!block_tree_fits((int)h.factor.size())) {
+        delete P;
+        return fail(c, MBC_UNSUPPORTED, "the plan's block entries do not fit shared memory");
     }
     if (c->device >= 0 && !h.w.empty()) {
         cudaError_t e = cudaSetDevice(c->device);
@@ -186,32 +188,18 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
             chunk_unit.push_back(u);
         }
         chunk_unit.push_back(n_units);
-        bool real_w = true;
-        for (auto& x : h.w) real_w = real_w && x.imag() == 0.0;
-        // one device allocation: entries | unit_pre | unit_leaf | leaf_f | leaf_w | chunk_unit
+        // one device allocation: entries | unit_pre | unit_leaf | leaf records | chunk_unit
         size_t off = 0;
         auto place = [&](size_t bytes) { size_t o = off; off = (off + bytes + 255) / 256 * 256; return o; };
         const size_t o_e = place(entry.size() * 4), o_pre = place(h.unit_pre.size() * 2),
-                     o_ul = place(h.unit_leaf.size() * 4), o_lf = place(h.leaf_f.size() * 2),
-                     o_lw = place(real_w ? 0 : lw.size() * 8), o_lwd = place(real_w ? 0 : h.w.size() * 16),
-                     o_rf = place(real_w ? h.w.size() * 8 : 0), o_rd = place(real_w ? h.w.size() * 8 : 0), o_cu = place(chunk_unit.size() * 8);
+                     o_ul = place(h.unit_leaf.size() * 4), o_rf = place(h.w.size() * 8), o_rd = place(h.w.size() * 8),
+                     o_cu = place(chunk_unit.size() * 8);
         std::vector<unsigned char> blob(std::max<size_t>(off, 256));
         std::memcpy(blob.data() + o_e, entry.data(), entry.size() * 4);
         if (!h.unit_pre.empty()) std::memcpy(blob.data() + o_pre, h.unit_pre.data(), h.unit_pre.size() * 2);
         std::memcpy(blob.data() + o_ul, h.unit_leaf.data(), h.unit_leaf.size() * 4);
-        std::memcpy(blob.data() + o_lf, h.leaf_f.data(), h.leaf_f.size() * 2);
-        if (!real_w) std::memcpy(blob.data() + o_lw, lw.data(), lw.size() * 8);
         for (size_t i = 0; i < h.w.size(); ++i) {
-            const double wd[2] = {h.w[i].real(), h.w[i].imag()};
-            if (!real_w) {
-                std::memcpy(blob.data() + o_lwd + 16 * i, wd, 16);
-                continue;
-            }
-            uint64_t bits;
-            std::memcpy(&bits, wd, 8);
-            uint32_t rf[2] = {h.leaf_f[i], 0u};
-            const uint32_t rd[2] = {h.leaf_f[i], (uint32_t)(bits >> 32)};
-            std::memcpy(rf + 1, &lw[i].x, 4);
+            const uint32_t rf[2] = {h.leaf_f[i], lw[i][0]}, rd[2] = {h.leaf_f[i], lw[i][1]};
             std::memcpy(blob.data() + o_rf + 8 * i, rf, 8);
             std::memcpy(blob.data() + o_rd + 8 * i, rd, 8);
         }
@@ -229,10 +217,6 @@ mbc_status mbc_block_plan_create(mbc_ctx* c, int op, int prec, mbc_block_plan** 
         P->td.n_units = n_units;
         P->td.unit_pre = reinterpret_cast<const uint16_t*>(base + o_pre);
         P->td.unit_leaf = reinterpret_cast<const int32_t*>(base + o_ul);
-        P->td.leaf_f = reinterpret_cast<const uint16_t*>(base + o_lf);
-        P->td.leaf_w = reinterpret_cast<const float2*>(base + o_lw);
-        P->td.leaf_wd = reinterpret_cast<const double2*>(base + o_lwd);
-        P->td.real_w = real_w ? 1 : 0;
         P->td.leaf_rf = reinterpret_cast<const uint2*>(base + o_rf);
         P->td.leaf_rd = reinterpret_cast<const uint2*>(base + o_rd);
         P->td.n_chunks = (int)n_chunks;
