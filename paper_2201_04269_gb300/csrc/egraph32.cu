@@ -668,29 +668,6 @@ constexpr double kSliceErr = 2.5e-7;
 constexpr int kGuardThreads = 512;
 constexpr int kGuardKeys = 40960;       // largest slice whose keys are kept in shared memory
 
-// Sum of one complex double per thread, valid in thread 0: each thread's value through shared
-// memory, warp 0 adds the real and warp 1 the imaginary parts (every 32nd value per lane, then a
-// shuffle tree), compensated.  buf: blockDim values; red: 4 doubles.  At least two warps.
-__device__ __forceinline__ void guard_sum(cd v, kacc& re, kacc& im, cd* buf, double* red) {
-    buf[threadIdx.x] = v;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp < 2) {
-        kacc k = {0.0, 0.0};
-        for (int i = lane; i < (int)blockDim.x; i += 32) kacc_add(k, warp == 0 ? buf[i].re : buf[i].im);
-        for (int off = 16; off > 0; off >>= 1) kacc_merge(k, kacc_shfl_down(k, off));
-        if (lane == 0) {
-            red[2 * warp] = k.hi;
-            red[2 * warp + 1] = k.lo;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        re = kacc{red[0], red[1]};
-        im = kacc{red[2], red[3]};
-    }
-}
-
 __device__ __forceinline__ void slice_guard_body(const d4* __restrict__ part, const double* __restrict__ scale,
                                                  int64_t st, int64_t V3, Momentum mom, double tol, int64_t unit0,
                                                  unsigned int* __restrict__ flag_count,
@@ -729,7 +706,7 @@ __device__ __forceinline__ void slice_guard_body(const d4* __restrict__ part, co
     }
     if (lane == 0) wsum[0][warp] = top;
     kacc kr, ki;
-    guard_sum(cd_make(re, im), kr, ki, buf, red);     // (its barriers order wsum too)
+    block_sum(cd_make(re, im), kr, ki, red, buf);     // (its barriers order wsum too)
     if (threadIdx.x == 0) {
         for (int w = 1; w < nw; ++w) top = top > wsum[0][w] ? top : wsum[0][w];
         s_max = top;
@@ -750,7 +727,7 @@ __device__ __forceinline__ void slice_guard_body(const d4* __restrict__ part, co
         q += r * r;
     }
     kacc kq, kz;
-    guard_sum(cd_make(q, 0.0), kq, kz, buf, red);
+    block_sum(cd_make(q, 0.0), kq, kz, red, buf);
     if (threadIdx.x == 0) {
         const double cr = kr.hi + kr.lo, ci = ki.hi + ki.lo;
         const double cabs = sqrt(cr * cr + ci * ci);
