@@ -296,7 +296,8 @@ mbc_status mbc_tensor_egraph(mbc_ctx* ctx, const char* expression, const char* a
  * first untimed), keeps the fastest in the plan and in the context's cache keyed by the
  * plan signature (a plan made later with the same signature starts from it), and reports
  * it.  Candidates that do not fit or fail to launch are skipped; on an error the plan
- * keeps its original schedule.  Synchronises the stream.
+ * keeps its original schedule.  A tree plan whose minors all follow from shared Laplace
+ * steps has no other candidate.  Synchronises the stream.
  *
  * For an MBC_PREC_FP32 e-graph plan the schedule is the FP32 kernel's shape: threads =
  * 128 x walkers (128..768; a walker is a group of 128 threads walking its part of the

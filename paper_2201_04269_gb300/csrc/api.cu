@@ -1622,8 +1622,11 @@ mbc_status mbc_autotune(mbc_plan* P, const void* U, const void* D, int64_t n_sit
         return a.threads == b.threads && a.blocks_per_sm == b.blocks_per_sm && a.sites_per_unit == b.sites_per_unit;
     };
     // candidates: the plan's current (default) schedule first, then the grid of block
-    // sizes x blocks per SM (x sites per unit for the direct sweep); for an FP32 plan the
+    // sizes x blocks per SM (x sites per unit for the direct sweep; for a tree block sizes of its
+    // LU kernel alone, and none where no flavour takes it); for an FP32 plan the
     // grid of kernel shapes, walkers x blocks per site x leaf batch
+    bool tree_lu = false;
+    for (int f = 0; f < 2; ++f) tree_lu = tree_lu || (P->td.n_minors[f] > 0 && !P->td.levels[f].n);
     std::vector<mbc_schedule> cands{orig};
     if (fp32) {
         for (int w : {3, 4, 5, 6})
@@ -1632,7 +1635,7 @@ mbc_status mbc_autotune(mbc_plan* P, const void* U, const void* D, int64_t n_sit
                     const mbc_schedule cand{128 * w, cs, lb};
                     if (!same(cand, orig)) cands.push_back(cand);
                 }
-    } else {
+    } else if (tree_lu || P->hp.algo != MBC_ALGO_TREE) {
         const int smem = P->ed.smem_values * 16 + 1024;
         for (int th : {128, 256, 320, 352, 384})
             for (int bps : {1, 2, 3, 4, 6, 8}) {

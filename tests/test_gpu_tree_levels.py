@@ -83,3 +83,25 @@ def test_tree_of_more_sites_than_one_wave(ctx, prec):
     parts = np.concatenate([sites(a, min(a + 300, n)) for a in range(0, n, 300)])
     plan.destroy()
     assert np.all(whole != 0) and np.array_equal(whole, parts)
+
+
+def test_tree_autotune_times_what_the_schedule_changes(ctx):
+    """The schedule sets the block size of the tree's LU kernel: a plan without it (dinucleon I) is
+    evaluated under its own schedule only, four times; one with it (the proton's down entries)
+    under others too."""
+    from paper_2201_04269_gb300 import abi
+    for op, alone in (("dinucleon_I", True), ("proton", False)):
+        plan = ctx.plan_operator(op, "tree", "mixed")
+        before = abi.mbc_get_schedule(plan.handle)
+        f = np.random.default_rng(9).standard_normal((2, 1, 1, 33, 12, 12, 2)).view(np.complex128)[..., 0]
+        U, D = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in f)
+        C = torch.zeros(1, 1, dtype=torch.complex128, device="cuda")
+        plan.correlator(U, D, C)
+        n0 = ctx.launches
+        plan.correlator(U, D, C)
+        n1 = ctx.launches
+        best = plan.autotune(U, D, 33)
+        evaluations = (ctx.launches - n1) / (n1 - n0)
+        assert evaluations == 4 if alone else evaluations > 4
+        assert not alone or best == before
+        plan.destroy()
