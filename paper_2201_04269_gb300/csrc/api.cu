@@ -707,8 +707,9 @@ mbc_status upload(mbc_plan* P, const MinorLevels (&ml)[2]) {
     const bool fused = compact && ed.n_j <= 2;
     const int base = 2 * kBlk + ed.stack_a + ed.stack_b + (fused ? 0 : ed.n_j * ed.n_rows_b);
     // the packed tables of the two leaf levels (uint32 words, in 16-byte units) go to shared
-    // memory too when that costs no resident block at 384 threads (the double-float kernel
-    // is issue-bound and needs the warps), and always for FP64 (bound by the FP64 pipe,
+    // memory too when that costs none of the five blocks that 384 threads allow (the double-float kernel
+    // is issue-bound and needs the warps; the plans of smaller blocks, with up to 18 per SM, have
+    // tables of a few hundred bytes), and always for FP64 (bound by the FP64 pipe,
     // it gains more from the shorter table reads than it loses in occupancy)
     const int pk16 = (ed.A.size[ed.A.n] * ed.A.n + ed.B.size[ed.B.n] * ed.B.n + 3) / 4;
     auto resident = [](int values) { return std::min(225 * 1024 / (values * 16 + 3 * 1024), 2048 / 384); };
@@ -798,9 +799,12 @@ mbc_status finish_plan(mbc_ctx* ctx, mbc_plan* P, mbc_plan** out) {
     P->signature = signature(h);
     if (h.algo == MBC_ALGO_EGRAPH) {
         // 384 threads (12 warps) per block, or the row-set counts rounded up to whole warps when these are
-        // smaller (one row set per thread in the leaf stage, no idle warp in its barriers), as
-        // many blocks per SM as shared memory, the registers (56 a thread) and the 2048-thread
-        // limit allow.  Against 384 threads, 8192 sites: dinucleon I double-float 13.95 -> 10.78 ms and
+        // smaller (one row set per thread in the leaf stage, no idle warp in its barriers); as
+        // many blocks per SM as shared memory and the 2048-thread limit allow, and of small blocks
+        // as the registers hold (56 a thread).  Up to five are launched in any case, of which
+        // three are resident at 320 threads or more (four in the FP64 build of 40 registers): the others
+        // start as these end, each with its K slot.
+        // Against 384 threads, 8192 sites: dinucleon I double-float 13.95 -> 10.78 ms and
         // FP64 28.6 -> 27.4 ms, proton 1020 -> 412 us and 1335 -> 609 us
         const int rows_w = (P->ed.n_rows_b + 31) / 32 * 32;
         const int rows_a = (P->ed.A.size[P->ed.A.n] + 31) / 32 * 32;
@@ -871,7 +875,7 @@ mbc_status run(mbc_plan* P, const void* U, const void* D, int n_sets, int T, int
         if (st != MBC_OK) return st;
         e = launch_tree(P->td, h.prec, u, d, g, c->scratch.p, wave, (int*)c->exps.p, parts, P->sched.threads, s, &c->launches);
     } else if (h.prec == MBC_PREC_FP32) {
-        // FP32 pass (one block per SM, a B table per block), then the double-float
+        // FP32 pass (one or two blocks per SM, a B table per block), then the double-float
         // kernel over the sites whose error estimate exceeded the guard
         const int grid32 = c->sms * P->e32.blocks;
         const int grid_df = (int)std::min<int64_t>(n_sites, (int64_t)c->sms * P->sched_df.blocks_per_sm);

@@ -251,7 +251,7 @@ struct Momentum {
     int L = 1, px = 0, py = 0, pz = 0;
     __host__ __device__ bool nonzero() const { return (px | py | pz) != 0; }
 };
-// FP32 e-graph kernel (egraph32.cu): one block per SM, one site per cluster of d.cs
+// FP32 e-graph kernel (egraph32.cu): d.blocks blocks per SM, one site per cluster of d.cs
 // blocks at a time, at most max_grid blocks; then the slice guard (unless slice_tol is
 // +inf).  Writes every site's partial and its error scale (scale, [n_sites] double, 0
 // for a site already listed); sites whose error estimate exceeds site_guard, and the
