@@ -149,8 +149,9 @@ typedef struct {
     int64_t minors_u, minors_d;  /* distinct minors the canonical form needs */
     int64_t tree_nodes;          /* vertices of the linearised factor tree (root included) */
     int64_t egraph_classes, egraph_nodes;     /* saturated minor e-graph size */
-    double flops_per_site;       /* algorithmic flops of this plan's algorithm, per site (tree: one LU
-                                    per minor; the kernels share Laplace steps between minors) */
+    double flops_per_site;       /* algorithmic flops of this plan's algorithm, per site: 8 per complex
+                                    multiply-add, 4 with a real weight (tree: the shared Laplace steps of
+                                    its minors, or one LU per minor where a flavour takes that, and the walk) */
     double direct_flops_per_site;/* the direct sweep's flops, per site (for comparison) */
     int64_t scratch_bytes_per_site; /* device scratch the algorithm uses per in-flight site */
 } mbc_plan_info;

@@ -44,6 +44,7 @@ struct mbc_plan {
     DirectDev dd{};
     TreeDev td{};
     int64_t tree_extra_rows = 0;  // rows of a tree plan's table below its minors
+    double tree_flops = 0;        // a tree plan's flops per site as its kernels take them
     EgraphDev ed{};
     Eg32Dev e32{};                // FP32 e-graph view (MBC_PREC_FP32 plans)
     void* dev32 = nullptr;        // its arrays (walk programs, packed words, G and pair records)
@@ -739,6 +740,18 @@ int64_t tree_levels(const HostPlan& h, MinorLevels (&ml)[2]) {
     return ml[0].n || ml[1].n ? extra + 288 : 0;           // 288: the entries of both flavours
 }
 
+// Flops of one site through the tree's kernels: Laplace levels (or an LU per minor), leaves with
+// their real or complex coefficients, level-1 products.
+double tree_flops(const HostPlan& h, const MinorLevels (&ml)[2]) {
+    const int nf[2] = {h.n_u, h.n_d};
+    double n = 8.0 * (double)h.tree.n_level1;
+    for (int f = 0; f < 2; ++f)
+        n += ml[f].n ? 8.0 * ml[f].cfma : (double)h.tree.minor_rows[f].size() * flops_lu(nf[f]);
+    bool real = true;
+    for (auto& x : h.tree.coefficients) real = real && x.imag() == 0.0;
+    return n + (real ? 4.0 : 8.0) * (double)h.tree.coefficients.size();
+}
+
 std::string signature(const HostPlan& h) {
     // identifies the plan's kernel workload for the autotune cache
     char buf[256];
@@ -768,6 +781,7 @@ mbc_status finish_plan(mbc_ctx* ctx, mbc_plan* P, mbc_plan** out) {
     MinorLevels ml[2];
     try {
         P->tree_extra_rows = tree_levels(h, ml);
+        P->tree_flops = tree_flops(h, ml);
     } catch (const std::bad_alloc&) {
         delete P;
         return fail(ctx, MBC_OOM, "host allocation while planning the tree's minors");
@@ -1120,7 +1134,7 @@ mbc_status mbc_plan_get_info(const mbc_plan* P, mbc_plan_info* info) {
     info->tree_nodes = (int64_t)h.tree.factors.size();
     info->egraph_classes = h.eg.A.classes + h.eg.B.classes;
     info->egraph_nodes = h.eg.A.enodes + h.eg.B.enodes;
-    info->flops_per_site = h.algo == MBC_ALGO_DIRECT ? h.flops_direct : (h.algo == MBC_ALGO_TREE ? h.flops_tree : h.flops_egraph);
+    info->flops_per_site = h.algo == MBC_ALGO_DIRECT ? h.flops_direct : (h.algo == MBC_ALGO_TREE ? P->tree_flops : h.flops_egraph);
     info->direct_flops_per_site = h.flops_direct;
     info->scratch_bytes_per_site = h.algo == MBC_ALGO_TREE ? ((int64_t)(h.tree.minor_rows[0].size() + h.tree.minor_rows[1].size()) + P->tree_extra_rows) * 16 : 32;
     return MBC_OK;

@@ -395,6 +395,22 @@ def test_minor_egraph_size_and_flops(abi, hctx, name):
     abi.mbc_plan_destroy(tree_plan)
 
 
+def test_tree_flops_are_those_of_its_kernels(abi, hctx):
+    """A tree plan's flops: the proton's up minors (2 x 2) cost two complex multiply-adds each, its down
+    minors nothing; with larger minors the shared Laplace steps cost less than one LU per minor."""
+    plan, _ = plan_of(abi, hctx, "proton", "tree")
+    info = abi.mbc_plan_get_info(plan)
+    level1 = info["tree_nodes"] - 1 - info["canonical_terms"]
+    assert info["flops_per_site"] == 8 * (2 * info["minors_u"] + level1) + 4 * info["canonical_terms"]
+    abi.mbc_plan_destroy(plan)
+    for name, lu in (("dinucleon_I", (86.0, 86.0)), ("he3_I", (356.0, 190.0))):
+        plan, _ = plan_of(abi, hctx, name, "tree")
+        info = abi.mbc_plan_get_info(plan)
+        walk = 8 * (info["tree_nodes"] - 1 - info["canonical_terms"]) + 4 * info["canonical_terms"]
+        assert walk < info["flops_per_site"] < walk + 0.6 * (info["minors_u"] * lu[0] + info["minors_d"] * lu[1])
+        abi.mbc_plan_destroy(plan)
+
+
 def test_fp32_plan_settings_on_the_host(abi, hctx):
     """MBC_PREC_FP32 plans on a host-only context: FP32 is accepted only for the e-graph
     algorithm; guard settings round-trip (NaN rejected); kernel shapes are validated

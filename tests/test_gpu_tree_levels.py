@@ -62,7 +62,7 @@ def test_tree_levels_match_direct(ctx, n_u, n_d, n_sets, n_terms, complex_w, pre
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_tree_of_more_sites_than_one_wave(ctx, prec):
-    """The tables of 3He I take 3.1 MB a site, so that 1500 sites run in three waves of at most 2 GB
+    """The tables of 3He I take 4 MB a site, so that 1500 sites run in three waves of at most 2 GB
     with a shorter last one: the same site values, bit for bit, as in calls of one wave each."""
     rng = np.random.default_rng(8)
     plan = ctx.plan_operator("he3_I", "tree", prec)
