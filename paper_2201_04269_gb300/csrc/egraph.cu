@@ -335,11 +335,13 @@ __global__ void __launch_bounds__(384, MIN_BLOCKS) egraph_kernel(EgraphDev d, co
 }
 
 // Several (plan, fields) items in one persistent launch: work units are (item, site),
-// numbered item by item; a block takes the unit of its own number, then units from the counter,
-// finds the item by a search over the unit offsets and evaluates the site with that item's
-// plan.  (Neighbouring blocks start on different SMs, so the units of a heavy item spread evenly; when
-// the first units came from the counter too, an SM of several small blocks could draw five of
-// them: dinucleon I and proton, 343 sites each in FP64, 2608 -> 1651 us.)  Three
+// numbered item by item; a block takes the unit of its own number, then units from the counter
+// (list mode: all from the counter), finds the item by a search over the unit offsets and
+// evaluates the site with that item's plan.  Neighbouring blocks start on different SMs, so the
+// units of a heavy item spread evenly; when the first units came from the counter too, an SM of
+// several small blocks could draw five of them: dinucleon I and proton, 343 sites each in FP64 2512 ->
+// 1662 us, in double-float 1242 -> 947 us.  (Large double-float batches take 0.3 to 0.9 % longer by the compiler's
+// allocation.)  Three
 // resident blocks of 384 threads per SM: the register cap this implies (56) costs a
 // few spills of the per-item plan view, which the occupancy more than repays.
 template <class P>
@@ -351,13 +353,18 @@ __global__ void __launch_bounds__(384, 3) egraph_batch_kernel(const BatchItem* _
                                                            int64_t n_units_list) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[4 * 32];
-    __shared__ unsigned int s_unit;
+    __shared__ unsigned int s_unit, s_first;
     const uint32_t* pk_owner = nullptr;
     typename P::V* K = kscratch + (size_t)blockIdx.x * kslot_values;
     // every unit, or (list mode) the units of a device list
     const int64_t n_work = list ? (int64_t)*list_n : n_units;
-    for (bool first = true;; first = false) {
-        if (threadIdx.x == 0) s_unit = first ? blockIdx.x : gridDim.x + atomicAdd(counter, 1u);
+    if (threadIdx.x == 0) s_first = list ? ~0u : blockIdx.x;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const unsigned int u = s_first;
+            s_unit = u != ~0u ? u : (list ? 0u : gridDim.x) + atomicAdd(counter, 1u);
+            s_first = ~0u;
+        }
         __syncthreads();
         const int64_t work = s_unit;
         if (work >= n_work) break;
@@ -386,7 +393,12 @@ cudaError_t launch_egraph_batch(const BatchItem* items, int n_items, int64_t n_u
     if (prec == 0) e = cudaFuncSetAttribute(egraph_batch_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     else e = cudaFuncSetAttribute(egraph_batch_kernel<MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgraphSmemMax);
     if (e != cudaSuccess) return e;
-    grid = (int)std::min<int64_t>(n_units, grid);
+    // no more blocks than are resident at the kernel's 56 registers: one that starts late would take the
+    // unit of its number last
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    grid = (int)std::min<int64_t>(n_units, std::min(grid, sms * (65536 / (56 * threads))));
     e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
     if (prec == 0)
